@@ -424,8 +424,15 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     }
   }
   const size_t need = (a.flags & APSP_FLAG_NO_WORKSPACE) ? 0 : workspace_bytes_with(n, dtype, a.S, a.flags);
-  if (need) {
-    if (opt && opt->workspace) {
+  const int R = (int)((n + a.S - 1) / a.S);
+  const size_t stage_need =
+      dtype != APSP_I16 && uses_stage_launches(a.S, R, a.flags, a.events != nullptr) ? stage_ws_bytes(R) : 0;
+  if (need || stage_need) {
+    if (opt && opt->workspace && !need) {
+      // not asked for: taken if it serves the one-launch-per-stage schedule
+      a.ws = opt->workspace;
+      a.ws_bytes = (size_t)std::max<int64_t>(opt->workspace_bytes, 0);
+    } else if (opt && opt->workspace) {
       // one panel buffer is enough (plain schedule); two allow the lookahead
       if (opt->workspace_bytes < (int64_t)panel_bytes_for(n, dtype, a.S) ||
           reinterpret_cast<uintptr_t>(opt->workspace) % 256)
@@ -433,7 +440,8 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       a.ws = opt->workspace;
       a.ws_bytes = (size_t)opt->workspace_bytes;
     } else {
-      a.ws = library_workspace(dev, a.stream, need, cap != cudaStreamCaptureStatusNone, &a.ws_bytes);
+      a.ws = library_workspace(dev, a.stream, std::max(need, stage_need), cap != cudaStreamCaptureStatusNone,
+                               &a.ws_bytes);
       if (!a.ws) a.ws_bytes = 0;  // the kernels fall back to the form that needs none
     }
   }

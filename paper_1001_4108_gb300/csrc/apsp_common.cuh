@@ -13,6 +13,7 @@ namespace apsp {
 enum DeviceError : int {
   kDevOk = 0,
   kDevTimeoutTma = 1,  // an mbarrier wait for a TMA copy gave up
+  kDevTimeoutFlag = 2, // a wait for another CTA's flag gave up
 };
 
 // Longest a bounded device wait spins before giving up (nanoseconds).

@@ -6,6 +6,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "../../include/apsp.h"
+
 namespace apsp {
 
 struct RunArgs {
@@ -78,6 +80,17 @@ constexpr int kStripMaxRoundsF32 = 48, kStripMaxRoundsI32 = 32;
 inline bool uses_strips(int S, int R, bool f32, bool i16) {
   return S == 64 && !i16 && R >= 2 && R <= (f32 ? kStripMaxRoundsF32 : kStripMaxRoundsI32);
 }
+
+// One launch per stage (stage.cuh), s = 64: calls without special requests
+// (no forced kernel, plain schedule or tracing) and enough workspace.
+constexpr int kStageMaxRounds = 32;
+inline bool uses_stage_launches(int S, int R, int flags, bool traced) {
+  constexpr int kOther = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_LOOKAHEAD | APSP_FLAG_NO_WORKSPACE;
+  return S == 64 && R <= kStageMaxRounds && !(flags & kOther) && !traced;
+}
+// Its workspace: two panel buffers (row and column, R tiles of 64 x 64 words
+// each) and two diagonal tiles.
+inline size_t stage_ws_bytes(int R) { return ((size_t)4 * R + 2) * 64 * 64 * sizeof(int32_t); }
 
 // Workspace bytes of the packed int16x2 phase 3 (replicated column panel:
 // n_p rows x s words).

@@ -53,8 +53,6 @@ namespace {
 
 constexpr int kDS = 64, kDM = 4;  // tile side, register block per thread
 using DShape = BShape<kDS, kDM>;  // 256 threads, padded shared rows
-// Device error code of a dataflow wait that gave up (the TMA waits use 1).
-constexpr int kDevTimeoutFlag = 2;
 
 __device__ __forceinline__ int ld_acquire(const int *p) {
   int v;
@@ -77,7 +75,7 @@ __device__ bool wait_geq(const int *p, int v, int *err) {
     if (ld_acquire(p) >= v) return true;
     if (*reinterpret_cast<volatile int *>(err) != 0) return false;
     if (globaltimer_ns() - t0 > kWaitLimitNs) {
-      atomicCAS(err, 0, kDevTimeoutFlag);
+      atomicCAS(err, 0, (int)kDevTimeoutFlag);
       return false;
     }
     __nanosleep(32);

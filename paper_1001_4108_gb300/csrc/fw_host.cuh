@@ -8,6 +8,8 @@
 #include "apsp_internal.h"
 #include "fw_kernels.cuh"
 #include "fw_s16x2.cuh"
+#include "launch.cuh"
+#include "stage.cuh"
 
 #include <type_traits>
 
@@ -106,35 +108,6 @@ struct Kernels {
   }
 };
 
-// Launches `k` on `st` as a programmatic dependent launch (see
-// wait_prior_grid); prio != 0 sets the launch's scheduling priority (both
-// are recorded in the node when the stream is being captured).
-template <typename... KP, typename... Args>
-static cudaError_t launch(void (*k)(KP...), dim3 grid, int threads, size_t smem, cudaStream_t st, int prio,
-                          Args... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[2];
-  unsigned na = 0;
-#if APSP_PDL
-  // every kernel launched here starts with wait_prior_grid()
-  at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[na].val.programmaticStreamSerializationAllowed = 1;
-  ++na;
-#endif
-  if (prio != 0) {
-    at[na].id = cudaLaunchAttributePriority;
-    at[na].val.priority = prio;
-    ++na;
-  }
-  cfg.attrs = na ? at : nullptr;
-  cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, k, args...);
-}
-
 // The stages of Fig. 2 for one matrix.
 //
 // Plain schedule, per stage b on the caller's stream: phase 1, phase 2,
@@ -208,6 +181,12 @@ static int run_rounds(const RunArgs &a) {
       const int dt = std::is_same<T, float>::value ? APSP_F32 : std::is_same<T, int16_t>::value ? APSP_I16 : APSP_I32;
       return run_dataflow(a, dt, static_cast<int *>(a.ws));
     }
+  }
+  // s = 64 without special requests: one launch per stage
+  if constexpr (S == 64 && HAS_TMA) {
+    if (uses_stage_launches(S, R, a.flags, a.events != nullptr) && a.ws && a.ws_bytes >= stage_ws_bytes(R) &&
+        reinterpret_cast<uintptr_t>(a.ws) % 256 == 0)
+      return run_stages<T, VIA>(a);
   }
   const cudaStream_t st = a.stream;
   const int64_t np = (int64_t)R * S;

@@ -143,8 +143,8 @@ __global__ void __launch_bounds__((S / 8) * (S / 4), S == 128 ? 2 : 4)
 // 2*(R-1) CTAs: the first R-1 take the row panel tiles (b, J), the rest the
 // column panel tiles (I, b).  Shared memory holds the closed diagonal tile D
 // and the panel tile X.
-//   row panel:    x_ij <- min(x_ij, D_ik + x_kj)
-//   column panel: x_ij <- min(x_ij, x_ik + D_kj)
+//   row panel:    x_ij <- min(x_ij, min_k D_ik + x_kj)
+//   column panel: x_ij <- min(x_ij, min_k x_ik + D_kj)
 //
 // With bp != nullptr the row panel tiles are also stored, k-pair interleaved,
 // into bp: element (k, j) of the pivot row block goes to
@@ -178,33 +178,24 @@ __global__ void __launch_bounds__(NT) fw_phase2(T *__restrict__ d, int64_t n, in
     X[i * S + j] = okx ? Arith<T>::load(d[(r0 + i) * ld + c0 + j]) : Arith<T>::inf();
   }
   __syncthreads();
-  if (row_panel) {
-    for (int k = 0; k < S; ++k) {
-      const C xkj = X[k * S + j];
+  // the min-plus product with the closed diagonal tile, as in the staged
+  // kernels: the same sums, so the result does not depend on which kernel ran
+  C acc[E];
 #pragma unroll
-      for (int r = 0; r < E; ++r) {
-        const int i = i0 + RS * r;
-        X[i * S + j] = Arith<T>::relax(X[i * S + j], D[i * S + k], xkj);
-      }
-      __syncthreads();
-    }
-  } else {
-    for (int k = 0; k < S; ++k) {
-      const C dkj = D[k * S + j];
+  for (int r = 0; r < E; ++r) acc[r] = X[(i0 + RS * r) * S + j];
+  const C *A = row_panel ? D : X, *B = row_panel ? X : D;
+#pragma unroll 4
+  for (int k = 0; k < S; ++k) {
+    const C bkj = B[k * S + j];
 #pragma unroll
-      for (int r = 0; r < E; ++r) {
-        const int i = i0 + RS * r;
-        X[i * S + j] = Arith<T>::relax(X[i * S + j], X[i * S + k], dkj);
-      }
-      __syncthreads();
-    }
+    for (int r = 0; r < E; ++r) acc[r] = Arith<T>::relax(acc[r], A[(i0 + RS * r) * S + k], bkj);
   }
 #pragma unroll
   for (int r = 0; r < E; ++r) {
     const int i = i0 + RS * r;
     if (r0 + i < n && c0 + j < n) {
-      const C v = X[i * S + j];
-      if (via) note_via(via, via_ld, r0 + i, c0 + j, v, Arith<T>::load(d[(r0 + i) * ld + c0 + j]), b);
+      const C v = acc[r];
+      if (via) note_via(via, via_ld, r0 + i, c0 + j, v, X[i * S + j], b);
       d[(r0 + i) * ld + c0 + j] = last ? Arith<T>::finish(v) : (T)v;
     }
   }
@@ -212,7 +203,7 @@ __global__ void __launch_bounds__(NT) fw_phase2(T *__restrict__ d, int64_t n, in
 #pragma unroll
     for (int r = 0; r < E; ++r) {
       const int i = i0 + RS * r;
-      bp[(int64_t)(i >> 1) * bp_ld + 2 * (c0 + j) + (i & 1)] = (T)X[i * S + j];
+      bp[(int64_t)(i >> 1) * bp_ld + 2 * (c0 + j) + (i & 1)] = (T)acc[r];
     }
   }
 }

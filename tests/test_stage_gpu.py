@@ -1,0 +1,93 @@
+"""The s = 64 schedule of one head and one rest per stage (csrc/stage.cuh):
+bit-identical to the plain schedule for any leading dimension and alignment,
+and to the oracle for the integers.
+
+The stage counts are the edges of its ranges: one stage; head and rest in one
+launch up to 5 stages; panel strips 16, 32 and 64 wide up to 9, 24 and 32
+stages; beyond, the lookahead schedule.  Whole and ragged last stages."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+from paper_1001_4108_gb300 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def graph(dt, n, seed):
+    g = np.random.Generator(np.random.PCG64(seed))
+    if dt == "f32":  # sums are rounded: full 24-bit mantissas
+        w = (1.0 - g.random((n, n))).astype(np.float32)
+        w[g.random((n, n)) < 0.5] = np.inf
+    else:
+        p = g.integers(0, 51, n)
+        w = (g.integers(0, 951, (n, n)) + p[:, None] - p[None, :]).astype(np.int32)
+        w[g.random((n, n)) > 0.1] = 1 << 29
+    np.fill_diagonal(w, 0)
+    return w
+
+
+def on_device(w, ld, offset=0):
+    """The matrix in a larger buffer, `offset` elements in, -7 around it."""
+    n = w.shape[0]
+    t = torch.from_numpy(w)
+    buf = torch.full((n * ld + offset,), -7, dtype=t.dtype, device="cuda")
+    d = buf[offset:].view(n, ld)
+    d[:, :n] = t.cuda()
+    return d
+
+
+@pytest.mark.parametrize("dt", ["f32", "i32"])
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 127, 128, 129, 320, 321, 576, 577, 640, 1536, 1537, 1600, 2047, 2048, 2049])
+def test_stage_schedule_equals_plain(dt, n):
+    w = graph(dt, n, n)
+    ref = on_device(w, (n + 3) // 4 * 4)
+    binding.apsp_fw(ref, n, flags=binding.FLAG_NO_LOOKAHEAD | binding.FLAG_NO_GRAPH)
+    if dt == "i32" and n <= 1600:
+        np.testing.assert_array_equal(ref[:, :n].cpu().numpy(), oracle.fw_int32_conv(w))
+    for ld, offset in ((n, 0), ((n + 3) // 4 * 4, 0), (n + 1, 0), (n + 37, 3)):
+        d = on_device(w, ld, offset)
+        binding.apsp_fw(d, n)
+        torch.cuda.synchronize()
+        assert torch.equal(d[:, :n], ref[:, :n]), (ld, offset)
+        assert bool((d[:, n:] == -7).all())
+    assert binding.device_error() == 0
+
+
+@pytest.mark.parametrize("dt", ["f32", "i32"])
+@pytest.mark.parametrize("n", [64, 65, 200, 321, 577, 1000, 1537])
+def test_stage_schedule_paths(dt, n):
+    # the stage record and the distances, against the plain schedule's
+    w = graph(dt, n, n + 1)
+    a, b = on_device(w, n), on_device(w, n)
+    va, vb = (torch.empty((n, n), dtype=torch.int16, device="cuda") for _ in range(2))
+    binding.apsp_fw_paths(a, va)
+    binding.apsp_fw_paths(b, vb, flags=binding.FLAG_NO_LOOKAHEAD | binding.FLAG_NO_GRAPH)
+    torch.cuda.synchronize()
+    assert torch.equal(a, b) and torch.equal(va, vb)
+
+
+@pytest.mark.parametrize("n", [321, 1600])
+def test_stage_schedule_capture_and_replay(n):
+    # direct, the library's graph, its replay, and a user's capture
+    w = graph("i32", n, n + 2)
+    src = on_device(w, n)
+    ref = src.clone()
+    binding.apsp_fw(ref, flags=binding.FLAG_NO_LOOKAHEAD | binding.FLAG_NO_GRAPH)
+    s = torch.cuda.Stream()
+    d = torch.empty_like(src)
+    with torch.cuda.stream(s):
+        for _ in range(3):
+            d.copy_(src)
+            binding.apsp_fw(d, stream=s)
+            s.synchronize()
+            assert torch.equal(d, ref)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        binding.apsp_fw(d, stream=s)
+    d.copy_(src)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(d, ref)
