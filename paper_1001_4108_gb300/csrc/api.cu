@@ -290,6 +290,39 @@ size_t workspace_bytes_with(int64_t n, int dtype, int S, int flags) {
   return bytes;
 }
 
+// Pool of the aligned copies of unaligned matrices (solve()), one per device;
+// memory above the threshold goes back to the device when nothing uses it.
+constexpr uint64_t kCopyPoolKeep = 64ull << 20;
+cudaMemPool_t g_copy_pool[kMaxDev];
+
+// A buffer in stream order; nullptr if there is none to be had.
+void *copy_buffer(int dev, size_t bytes, cudaStream_t stream) {
+  cudaMemPool_t pool;
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (!g_copy_pool[dev]) {
+      cudaMemPoolProps props{};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      uint64_t keep = kCopyPoolKeep;
+      if (cudaMemPoolCreate(&g_copy_pool[dev], &props) != cudaSuccess ||
+          cudaMemPoolSetAttribute(g_copy_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        g_copy_pool[dev] = nullptr;
+        return nullptr;
+      }
+    }
+    pool = g_copy_pool[dev];
+  }
+  void *p = nullptr;
+  if (cudaMallocFromPoolAsync(&p, bytes, pool, stream) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return p;
+}
+
 // Device buffer of apsp_fw_host, one per device, grown on demand.
 struct HostStage {
   std::mutex mu;
@@ -453,7 +486,26 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
                                a.stream) != cudaSuccess)  // every entry -1: never improved
     return APSP_ECUDA;
   const bool direct = (a.flags & APSP_FLAG_NO_GRAPH) || a.events || cap != cudaStreamCaptureStatusNone;
-  st = direct ? run_dtype(a, dtype) : launch_with_graph(a, dtype, dev);
+  // Rows that are not 16-byte aligned: the staged kernels work on an aligned
+  // copy (two passes over the matrix, against kernels two to four times slower;
+  // the one-launch-per-stage schedule takes any layout by itself).
+  constexpr int kInPlace = APSP_FLAG_GENERIC | APSP_FLAG_NO_WORKSPACE;
+  const bool any_layout = stage_need && a.ws_bytes >= stage_need;
+  void *copy = nullptr;
+  const int64_t cld = (n * (int64_t)es + 15) / 16 * 16 / (int64_t)es;
+  if (!a.tma_ok && !any_layout && R > 1 && !(a.flags & kInPlace) && cap == cudaStreamCaptureStatusNone)
+    copy = copy_buffer(dev, (size_t)n * cld * es, a.stream);
+  if (copy) {
+    if (copy_matrix(dist, ld, copy, cld, n, (int)es, a.stream) != APSP_OK) st = APSP_ECUDA;
+    a.d = copy;
+    a.ld = cld;
+    a.tma_ok = true;
+  }
+  if (st == APSP_OK) st = direct ? run_dtype(a, dtype) : launch_with_graph(a, dtype, dev);
+  if (copy) {
+    if (st == APSP_OK && copy_matrix(copy, cld, dist, ld, n, (int)es, a.stream) != APSP_OK) st = APSP_ECUDA;
+    if (cudaFreeAsync(copy, a.stream) != cudaSuccess && st == APSP_OK) st = APSP_ECUDA;
+  }
   if (st != APSP_OK) return st;
   if (a.flags & APSP_FLAG_NEGCYCLE) return check_negcycle(dist, n, ld, dtype, a.stream, neg);
   return APSP_OK;

@@ -142,6 +142,7 @@ int run_i16(const RunArgs &a);
 int validate_input(const void *dist, int64_t n, int64_t ld, int dtype, cudaStream_t st, bool narrow);
 int check_negcycle(void *dist, int64_t n, int64_t ld, int dtype, cudaStream_t st, int *neg);
 int narrow_to_i16(const int32_t *src, int64_t n, int64_t ld, int16_t *dst, int64_t ld16, cudaStream_t st);
+int copy_matrix(const void *src, int64_t sld, void *dst, int64_t dld, int64_t n, int elem, cudaStream_t st);
 int widen_from_i16(const int16_t *src, int64_t ld16, int64_t n, int32_t *dst, int64_t ld, cudaStream_t st);
 
 // Tile side the C ABI picks for (n, dtype) when none is requested.

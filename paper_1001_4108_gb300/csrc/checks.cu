@@ -107,6 +107,13 @@ __global__ void widen_i16(const int16_t *src, int64_t ld16, int64_t n, int32_t *
       dst[i * ld + j] = v >= 16383 ? (1 << 29) : v;
     }
 }
+// n x n elements between matrices of different leading dimensions.
+template <typename T>
+__global__ void copy_rows(const T *src, int64_t sld, T *dst, int64_t dld, int64_t n) {
+  for (int64_t i = blockIdx.y; i < n; i += gridDim.y)
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
+      dst[i * dld + j] = src[i * sld + j];
+}
 dim3 rows_grid(int64_t n) {
   return dim3((unsigned)std::min<int64_t>((n + 255) / 256, 4), (unsigned)std::min<int64_t>(n, 4096));
 }
@@ -120,6 +127,16 @@ int narrow_to_i16(const int32_t *src, int64_t n, int64_t ld, int16_t *dst, int64
 
 int widen_from_i16(const int16_t *src, int64_t ld16, int64_t n, int32_t *dst, int64_t ld, cudaStream_t st) {
   widen_i16<<<rows_grid(n), 256, 0, st>>>(src, ld16, n, dst, ld);
+  return cudaPeekAtLastError() == cudaSuccess ? APSP_OK : APSP_ECUDA;
+}
+
+int copy_matrix(const void *src, int64_t sld, void *dst, int64_t dld, int64_t n, int elem, cudaStream_t st) {
+  if (elem == 2)
+    copy_rows<int16_t><<<rows_grid(n), 256, 0, st>>>(static_cast<const int16_t *>(src), sld,
+                                                     static_cast<int16_t *>(dst), dld, n);
+  else
+    copy_rows<int32_t><<<rows_grid(n), 256, 0, st>>>(static_cast<const int32_t *>(src), sld,
+                                                     static_cast<int32_t *>(dst), dld, n);
   return cudaPeekAtLastError() == cudaSuccess ? APSP_OK : APSP_ECUDA;
 }
 
