@@ -21,8 +21,7 @@ namespace {
 
 template <typename T, int S, int M>
 __global__ void __launch_bounds__(BShape<S, M>::NT, BShape<S, M>::MIN_BLOCKS)
-    fw_batched_cta(const BatchDesc *__restrict__ descs, int count,
-                                                                   int *counter) {
+    fw_batched_cta(const BatchDesc *__restrict__ descs, int count, int *counter, int one) {
   using C = typename Arith<T>::C;
   using IO = TileIO<T, S, M>;
   constexpr int LD = BShape<S, M>::LD;
@@ -65,9 +64,9 @@ __global__ void __launch_bounds__(BShape<S, M>::NT, BShape<S, M>::MIN_BLOCKS)
         __syncthreads();
         if (warp_has_work<M>(ty, tx, (int)min((int64_t)S, n - r0), (int)min((int64_t)S, n - c0))) {
           if (row)
-            minplus_tile<T, S, M>(acc, Ds, Ps, ty, tx, kq_end);
+            minplus_tile<T, S, M>(acc, Ds, Ps, ty, tx, kq_end, one);
           else
-            minplus_tile<T, S, M>(acc, Ps, Ds, ty, tx, kq_end);
+            minplus_tile<T, S, M>(acc, Ps, Ds, ty, tx, kq_end, one);
         }
         IO::store(d, ld, n, r0, c0, ty, tx, acc, last, vec);
         __syncthreads();
@@ -86,7 +85,7 @@ __global__ void __launch_bounds__(BShape<S, M>::NT, BShape<S, M>::MIN_BLOCKS)
           IO::to_smem(Qs, ty, tx, bt);
           __syncthreads();
           if (warp_has_work<M>(ty, tx, (int)min((int64_t)S, n - r0), (int)min((int64_t)S, n - c0)))
-            minplus_tile<T, S, M>(acc, Ps, Qs, ty, tx, kq_end);
+            minplus_tile<T, S, M>(acc, Ps, Qs, ty, tx, kq_end, one);
           IO::store(d, ld, n, r0, c0, ty, tx, acc, last, vec);
           __syncthreads();
         }
@@ -114,7 +113,7 @@ int launch_batched_kernel(const BatchDesc *descs, int count, int *counter, cudaS
     return APSP_ECUDA;
   const int grid = std::max(1, std::min(count, sms * std::max(per_sm, 1)));
   if (cudaMemsetAsync(counter, 0, sizeof(int), st) != cudaSuccess) return APSP_ECUDA;
-  fw_batched_cta<T, S, M><<<grid, B::NT, B::SMEM, st>>>(descs, count, counter);
+  fw_batched_cta<T, S, M><<<grid, B::NT, B::SMEM, st>>>(descs, count, counter, 1);
   return cudaPeekAtLastError() == cudaSuccess ? APSP_OK : APSP_ECUDA;
 }
 

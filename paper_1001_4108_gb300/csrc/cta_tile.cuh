@@ -8,6 +8,8 @@
 
 #include "apsp_common.cuh"
 
+#include <type_traits>
+
 #ifndef APSP_BATCH64_CTAS
 #define APSP_BATCH64_CTAS 3
 #endif
@@ -156,7 +158,7 @@ struct TileIO {
 // memory with the padded stride.
 template <typename T, int S, int M>
 __device__ __forceinline__ void minplus_tile(typename Arith<T>::C (&acc)[M][M], const typename Arith<T>::C *A,
-                                             const typename Arith<T>::C *B, int ty, int tx, int kq_end) {
+                                             const typename Arith<T>::C *B, int ty, int tx, int kq_end, int one) {
   using C = typename Arith<T>::C;
   constexpr int LD = BShape<S, M>::LD;
   static_assert(sizeof(C) == 4 && (M == 2 || M == 4), "vector shared loads of 4-byte elements");
@@ -173,24 +175,34 @@ __device__ __forceinline__ void minplus_tile(typename Arith<T>::C (&acc)[M][M], 
       av[a][3] = word_as<C>(v.w);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const C *q = B + (4 * kq + u) * LD + M * tx;
-      C bv[M];
-      if constexpr (M == 4) {
-        const int4 v = *reinterpret_cast<const int4 *>(q);
-        bv[0] = word_as<C>(v.x);
-        bv[1] = word_as<C>(v.y);
-        bv[2] = word_as<C>(v.z);
-        bv[3] = word_as<C>(v.w);
-      } else {
-        const int2 v = *reinterpret_cast<const int2 *>(q);
-        bv[0] = word_as<C>(v.x);
-        bv[1] = word_as<C>(v.y);
+    for (int u = 0; u < 4; u += 2) {  // two k's at a time
+      C bv[2][M];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const C *q = B + (4 * kq + u + e) * LD + M * tx;
+        if constexpr (M == 4) {
+          const int4 v = *reinterpret_cast<const int4 *>(q);
+          bv[e][0] = word_as<C>(v.x);
+          bv[e][1] = word_as<C>(v.y);
+          bv[e][2] = word_as<C>(v.z);
+          bv[e][3] = word_as<C>(v.w);
+        } else {
+          const int2 v = *reinterpret_cast<const int2 *>(q);
+          bv[e][0] = word_as<C>(v.x);
+          bv[e][1] = word_as<C>(v.y);
+        }
       }
 #pragma unroll
       for (int a = 0; a < M; ++a)
 #pragma unroll
-        for (int c = 0; c < M; ++c) acc[a][c] = Arith<T>::relax(acc[a][c], av[a][u], bv[c]);
+        for (int c = 0; c < M; ++c) {
+          if constexpr (std::is_same<C, float>::value)  // the two k's come in separate registers: scalar adds
+            acc[a][c] = min3f(acc[a][c], __fadd_rn(av[a][u], bv[0][c]), __fadd_rn(av[a][u + 1], bv[1][c]));
+          else if ((a + c) % 2 == 0)
+            acc[a][c] = relax2<true>(acc[a][c], av[a][u], av[a][u + 1], bv[0][c], bv[1][c], one);
+          else
+            acc[a][c] = relax2<false>(acc[a][c], av[a][u], av[a][u + 1], bv[0][c], bv[1][c], one);
+        }
     }
   }
 }

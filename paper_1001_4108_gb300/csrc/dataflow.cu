@@ -84,7 +84,7 @@ __device__ bool wait_geq(const int *p, int v, int *err) {
 
 template <typename T>
 __global__ void __launch_bounds__(DShape::NT, 2)
-    fw_dataflow(T *__restrict__ d, int64_t n, int64_t ld, int R, int *flags, int *err) {
+    fw_dataflow(T *__restrict__ d, int64_t n, int64_t ld, int R, int *flags, int *err, int one) {
   using C = typename Arith<T>::C;
   using IO = TileIO<T, kDS, kDM, true>;  // loads through L2: tiles come from other SMs
   constexpr int S = kDS, M = kDM, LD = DShape::LD;
@@ -156,9 +156,9 @@ __global__ void __launch_bounds__(DShape::NT, 2)
           __syncthreads();
           if (warp_has_work<M>(ty, tx, (int)min((int64_t)S, n - r0), (int)min((int64_t)S, n - c0))) {
             if (I == s)
-              minplus_tile<T, S, M>(acc, As, Bs, ty, tx, kq_end);  // row panel: D (x) X
+              minplus_tile<T, S, M>(acc, As, Bs, ty, tx, kq_end, one);  // row panel: D (x) X
             else
-              minplus_tile<T, S, M>(acc, Bs, As, ty, tx, kq_end);  // column panel: X (x) D
+              minplus_tile<T, S, M>(acc, Bs, As, ty, tx, kq_end, one);  // column panel: X (x) D
           }
           IO::store(d, ld, n, r0, c0, ty, tx, acc, last, vec);
         } else {
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(DShape::NT, 2)
           IO::to_smem(Bs, ty, tx, bt);
           __syncthreads();
           if (warp_has_work<M>(ty, tx, (int)min((int64_t)S, n - r0), (int)min((int64_t)S, n - c0)))
-            minplus_tile<T, S, M>(acc, As, Bs, ty, tx, kq_end);
+            minplus_tile<T, S, M>(acc, As, Bs, ty, tx, kq_end, one);
           IO::store(d, ld, n, r0, c0, ty, tx, acc, last, vec);
         }
         __syncthreads();  // the tile is stored and its operands read
@@ -210,7 +210,7 @@ int launch_dataflow(const RunArgs &a, int *flags) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   T *d = static_cast<T *>(a.d);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, fw_dataflow<T>, d, a.n, a.ld, R, flags, a.err);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, fw_dataflow<T>, d, a.n, a.ld, R, flags, a.err, 1);
   return e == cudaSuccess ? APSP_OK : APSP_ECUDA;
 }
 

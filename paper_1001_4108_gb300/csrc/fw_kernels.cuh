@@ -566,15 +566,6 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
 // blockIdx.x numbers the tiles of the launch's tile set.  FULL = true: every
 // row and column of every tile is inside the matrix (interior tiles); FULL =
 // false: masked loads/stores (the edge tiles of a ragged matrix).
-__device__ __forceinline__ float min3f(float a, float b, float c) {
-  float r;
-  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-
-// (a.x + b.x, a.y + b.y), each rounded to nearest: one packed add.f32x2.
-__device__ __forceinline__ float2 add2f(float2 a, float2 b) { return __fadd2_rn(a, b); }
-
 template <int S, bool REVERSE, bool FULL, bool VIA = false>
 __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
     fw_phase3_f32x2(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBp,

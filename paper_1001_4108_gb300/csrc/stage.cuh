@@ -65,6 +65,7 @@ struct StageArgs {
   int heads;         // head CTAs (a multiple of the cluster); in one launch with rest, its CTAs follow
   int rest;          // rest CTAs that update a tile
   int wait_first;    // rest: no head runs beside it
+  int one;           // 1 (relax2)
   C *ws;
   int16_t *via;
   int64_t via_ld;
@@ -74,15 +75,6 @@ struct StageArgs {
   __device__ __forceinline__ C *col_panel(int stage) const { return row_panel(stage) + (size_t)R * kStTile; }
   __device__ __forceinline__ C *diag(int stage) const { return ws + ((size_t)4 * R + (stage & 1)) * kStTile; }
 };
-
-// min(acc, a.x + b.x, a.y + b.y): two k's of one element.
-__device__ __forceinline__ float relax2(float acc, float a0, float a1, float b0, float b1) {
-  const float2 s = add2f(make_float2(a0, a1), make_float2(b0, b1));
-  return min3f(acc, s.x, s.y);
-}
-__device__ __forceinline__ int32_t relax2(int32_t acc, int32_t a0, int32_t a1, int32_t b0, int32_t b1) {
-  return __viaddmin_s32(a1, b1, __viaddmin_s32(a0, b0, acc));
-}
 
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -123,7 +115,7 @@ __device__ __forceinline__ int st_idx(int t, int a) { return 2 * t + 32 * (a >> 
 // at a + 64 m (m < M); B: rows of BS words, its column pairs at b + BSTEP q
 // (q < Q).
 template <typename C, int KP, int M, int Q, int AS, int BS, int BSTEP, int UN>
-__device__ __forceinline__ void st_product(C (&y)[2 * M][2 * Q], const C *a, const C *b, int kp0 = 0) {
+__device__ __forceinline__ void st_product(C (&y)[2 * M][2 * Q], const C *a, const C *b, int one, int kp0 = 0) {
   using V = typename Vec4<C>::V;
 #pragma unroll UN
   for (int i = 0; i < KP; ++i) {
@@ -137,10 +129,10 @@ __device__ __forceinline__ void st_product(C (&y)[2 * M][2 * Q], const C *a, con
     for (int m = 0; m < M; ++m)
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
-        y[2 * m][2 * q] = relax2(y[2 * m][2 * q], av[m].x, av[m].y, bv[q].x, bv[q].y);
-        y[2 * m][2 * q + 1] = relax2(y[2 * m][2 * q + 1], av[m].x, av[m].y, bv[q].z, bv[q].w);
-        y[2 * m + 1][2 * q] = relax2(y[2 * m + 1][2 * q], av[m].z, av[m].w, bv[q].x, bv[q].y);
-        y[2 * m + 1][2 * q + 1] = relax2(y[2 * m + 1][2 * q + 1], av[m].z, av[m].w, bv[q].z, bv[q].w);
+        y[2 * m][2 * q] = relax2<true>(y[2 * m][2 * q], av[m].x, av[m].y, bv[q].x, bv[q].y, one);
+        y[2 * m][2 * q + 1] = relax2<false>(y[2 * m][2 * q + 1], av[m].x, av[m].y, bv[q].z, bv[q].w, one);
+        y[2 * m + 1][2 * q] = relax2<false>(y[2 * m + 1][2 * q], av[m].z, av[m].w, bv[q].x, bv[q].y, one);
+        y[2 * m + 1][2 * q + 1] = relax2<true>(y[2 * m + 1][2 * q + 1], av[m].z, av[m].w, bv[q].z, bv[q].w, one);
       }
   }
 }
@@ -160,7 +152,7 @@ __device__ __forceinline__ void st_product(C (&y)[2 * M][2 * Q], const C *a, con
 // pivots: 2 x 1024 words (alternating between groups).
 template <typename T, typename F>
 __device__ __forceinline__ void st_close(typename Arith<T>::C (&x)[4][4], typename Arith<T>::C *pivots, int ty,
-                                         int tx, F &&beside) {
+                                         int tx, int one, F &&beside) {
   using C = typename Arith<T>::C;
   using V = typename Vec4<C>::V;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -216,7 +208,7 @@ __device__ __forceinline__ void st_close(typename Arith<T>::C (&x)[4][4], typena
         beside(4 * m + g);
       }
       __syncthreads();
-      st_product<C, 4, 2, 2, 128, 128, 64, 4>(x, cc + 4 * ty, rr + 4 * tx);
+      st_product<C, 4, 2, 2, 128, 128, 64, 4>(x, cc + 4 * ty, rr + 4 * tx, one);
     }
   }
 }
@@ -280,7 +272,7 @@ __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typenam
         }
       }
     const bool late = !mbar_wait_bounded(bar, 0);
-    if (!late) st_product<C, 32, 2, 2, 128, 128, 64, 4>(x, As + 4 * ty, Bs + 4 * tx);
+    if (!late) st_product<C, 32, 2, 2, 128, 128, 64, 4>(x, As + 4 * ty, Bs + 4 * tx, g.one);
     if (__any_sync(0xffffffffu, late)) {  // give up: wait (bounded) for the copies in flight, store nothing
       if (lane == 0) {
         atomicCAS(g.err, 0, (int)kDevTimeoutTma);
@@ -405,7 +397,7 @@ __global__ void __launch_bounds__(kStThreads) __cluster_dims__(kStCluster, 1, 1)
         t[e][f] = i < g.n && j < g.n ? Arith<T>::load(tsrc[i * tld + j]) : Arith<T>::inf();
       }
     late = !mbar_wait_bounded(&bar, 0);
-    if (!late) st_product<C, 32, 1, 1, 128, 128, 64, 8>(t, sm.a + 2 * r0, sm.b + 4 * lane);
+    if (!late) st_product<C, 32, 1, 1, 128, 128, 64, 8>(t, sm.a + 2 * r0, sm.b + 4 * lane, g.one);
     cluster_wait();  // the other CTAs have started: their shared memory can be written
 #pragma unroll
     for (int r = 0; r < kStCluster; ++r)
@@ -455,8 +447,8 @@ __global__ void __launch_bounds__(kStThreads) __cluster_dims__(kStCluster, 1, 1)
 
   // ---- phase 1 of stage c, with phase 3 of stage b on the strip beside it
   const C *ca = cols ? sm.b : sm.a;
-  st_close<T>(x, sm.pivots, ty, tx, [&](int k) {
-    if (upd) st_product<C, 4, 2, Q, 128, 2 * W, 32, 2>(y, ca + 4 * sy, sm.op + 4 * sx, 4 * k);
+  st_close<T>(x, sm.pivots, ty, tx, g.one, [&](int k) {
+    if (upd) st_product<C, 4, 2, Q, 128, 2 * W, 32, 2>(y, ca + 4 * sy, sm.op + 4 * sx, g.one, 4 * k);
   });
   if (lead) {
 #pragma unroll
@@ -519,7 +511,7 @@ __global__ void __launch_bounds__(kStThreads) __cluster_dims__(kStCluster, 1, 1)
 #pragma unroll
     for (int e = 0; e < 4; ++e) o[e & 1][2 * q + (e >> 1)] = z[e & 1][2 * q + (e >> 1)];
   }
-  st_product<C, 32, 1, Q, 128, 2 * W, 32, Q == 1 ? 8 : 4>(z, sm.form + 4 * ry, sm.strip + 4 * sx);
+  st_product<C, 32, 1, Q, 128, 2 * W, 32, Q == 1 ? 8 : 4>(z, sm.form + 4 * ry, sm.strip + 4 * sx, g.one);
 #pragma unroll
   for (int q = 0; q < Q; ++q)
     *reinterpret_cast<V *>(out + ry * 128 + 4 * sx + 32 * q) =
@@ -609,6 +601,7 @@ static int run_stages(const RunArgs &a) {
   g.via = a.via;
   g.via_ld = a.via_ld;
   g.err = a.err;
+  g.one = 1;
   const HeadCut cut = head_cut(R);
   g.half = std::max(1, S / cut.W * (R - 1));
   g.heads = (2 * g.half + kStCluster - 1) / kStCluster * kStCluster;
