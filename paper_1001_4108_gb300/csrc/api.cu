@@ -427,7 +427,10 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     const int64_t ld16 = (n + 7) / 8 * 8;
     const int S16 = choose_kblock(n, APSP_I16, opt ? opt->kblock : 0);
     const size_t copy_bytes = ((size_t)n * ld16 * 2 + 255) / 256 * 256;
-    const size_t ws16 = workspace_bytes_for(n, APSP_I16, S16);
+    const int R16 = (int)((n + S16 - 1) / S16);
+    size_t ws16 = workspace_bytes_for(n, APSP_I16, S16);
+    if (uses_stage_launches(S16, R16, true, a.flags, a.events != nullptr))
+      ws16 = std::max(ws16, stage_ws_bytes(R16));
     size_t got = 0;
     char *buf = static_cast<char *>(
         library_workspace(dev, a.stream, copy_bytes + ws16, cap != cudaStreamCaptureStatusNone, &got));
@@ -459,7 +462,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   const size_t need = (a.flags & APSP_FLAG_NO_WORKSPACE) ? 0 : workspace_bytes_with(n, dtype, a.S, a.flags);
   const int R = (int)((n + a.S - 1) / a.S);
   const size_t stage_need =
-      dtype != APSP_I16 && uses_stage_launches(a.S, R, a.flags, a.events != nullptr) ? stage_ws_bytes(R) : 0;
+      uses_stage_launches(a.S, R, dtype == APSP_I16, a.flags, a.events != nullptr) ? stage_ws_bytes(R) : 0;
   if (need || stage_need) {
     if (opt && opt->workspace && !need) {
       // not asked for: taken if it serves the one-launch-per-stage schedule

@@ -81,12 +81,17 @@ inline bool uses_strips(int S, int R, bool f32, bool i16) {
   return S == 64 && !i16 && R >= 2 && R <= (f32 ? kStripMaxRoundsF32 : kStripMaxRoundsI32);
 }
 
-// One launch per stage (stage.cuh), s = 64: calls without special requests
-// (no forced kernel, plain schedule or tracing) and enough workspace.
-constexpr int kStageMaxRounds = 32;
-inline bool uses_stage_launches(int S, int R, int flags, bool traced) {
+// One head and one rest per stage (stage.cuh), s = 64: calls without special
+// requests (no forced kernel, plain schedule or tracing) and enough workspace,
+// up to the stage count at which its rest stops paying.  us per solve with the
+// lookahead schedule and with it: int32 n = 1300 489 and 339, 1664 565 and 503,
+// 2048 776 and 778, 3072 about 2000 and 2080; fp32 n = 1408 445 and 403, 1792
+// 612 and 629, 2048 952 and 822.  int16 is computed in 32 bits here, half the
+// packed kernels' rate: n = 1024 296 and 229, 1280 375 and 328, 1408 406 and 413.
+constexpr int kStageMaxRounds = 32, kStageMaxRoundsI16 = 21;
+inline bool uses_stage_launches(int S, int R, bool i16, int flags, bool traced) {
   constexpr int kOther = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_LOOKAHEAD | APSP_FLAG_NO_WORKSPACE;
-  return S == 64 && R <= kStageMaxRounds && !(flags & kOther) && !traced;
+  return S == 64 && R <= (i16 ? kStageMaxRoundsI16 : kStageMaxRounds) && !(flags & kOther) && !traced;
 }
 // Its workspace: two panel buffers (row and column, R tiles of 64 x 64 words
 // each) and two diagonal tiles.

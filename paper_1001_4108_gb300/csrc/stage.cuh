@@ -213,6 +213,28 @@ __device__ __forceinline__ void st_close(typename Arith<T>::C (&x)[4][4], typena
   }
 }
 
+// Two adjacent elements, read through L2 only; and written.
+__device__ __forceinline__ void ld2cg(const float *p, float &x, float &y) {
+  const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
+  x = v.x;
+  y = v.y;
+}
+__device__ __forceinline__ void ld2cg(const int32_t *p, int32_t &x, int32_t &y) {
+  const int2 v = __ldcg(reinterpret_cast<const int2 *>(p));
+  x = v.x;
+  y = v.y;
+}
+__device__ __forceinline__ void ld2cg(const int16_t *p, int32_t &x, int32_t &y) {
+  const short2 v = __ldcg(reinterpret_cast<const short2 *>(p));
+  x = v.x;
+  y = v.y;
+}
+__device__ __forceinline__ void st2(float *p, float x, float y) { *reinterpret_cast<float2 *>(p) = make_float2(x, y); }
+__device__ __forceinline__ void st2(int32_t *p, int32_t x, int32_t y) { *reinterpret_cast<int2 *>(p) = make_int2(x, y); }
+__device__ __forceinline__ void st2(int16_t *p, int16_t x, int16_t y) {
+  *reinterpret_cast<short2 *>(p) = make_short2(x, y);
+}
+
 // rest(b): phase 3 of stage b on the tiles outside rows and columns b, c: CTA t
 // of g.rest updates one 64 x 64 tile, 4 x 4 elements per thread; one more CTA
 // (t = g.rest) moves the closed diagonal tile of stage b to the matrix.  As, Bs:
@@ -222,7 +244,6 @@ template <typename T, bool VIA>
 __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typename Arith<T>::C *As,
                                            typename Arith<T>::C *Bs, uint64_t *bar) {
   using C = typename Arith<T>::C;
-  using V2 = typename std::conditional<std::is_same<C, float>::value, float2, int2>::type;
   constexpr int S = kStS;
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const int b = g.b, R = g.R, c = b + 1;
@@ -252,9 +273,9 @@ __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typenam
     const int ty = 4 * (warp / 2) + lane / 8, tx = 8 * (warp % 2) + lane % 8;
     const int64_t i0 = (int64_t)I * S + 2 * ty, j0 = (int64_t)J * S + 2 * tx;
     const bool whole = (int64_t)(I + 1) * S <= g.n && (int64_t)(J + 1) * S <= g.n;
-    // whole tiles and rows that allow 8-byte accesses
-    const bool pair_in = whole && reinterpret_cast<uintptr_t>(g.src) % 8 == 0 && g.src_ld % 2 == 0;
-    const bool pair_out = whole && reinterpret_cast<uintptr_t>(g.dst) % 8 == 0 && g.dst_ld % 2 == 0;
+    // whole tiles and rows that allow two elements per access
+    const bool pair_in = whole && reinterpret_cast<uintptr_t>(g.src) % (2 * sizeof(T)) == 0 && g.src_ld % 2 == 0;
+    const bool pair_out = whole && reinterpret_cast<uintptr_t>(g.dst) % (2 * sizeof(T)) == 0 && g.dst_ld % 2 == 0;
     C x[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -263,16 +284,14 @@ __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typenam
         const int64_t i = i0 + st_idx(0, a), j = j0 + st_idx(0, e);
         const T *p = g.src + i * g.src_ld + j;
         if (pair_in) {
-          const V2 v = __ldcg(reinterpret_cast<const V2 *>(p));
-          x[a][e] = v.x;
-          x[a][e + 1] = v.y;
+          ld2cg(p, x[a][e], x[a][e + 1]);
         } else {
-          x[a][e] = i < g.n && j < g.n ? __ldcg(p) : Arith<T>::inf();
-          x[a][e + 1] = i < g.n && j + 1 < g.n ? __ldcg(p + 1) : Arith<T>::inf();
+          x[a][e] = i < g.n && j < g.n ? Arith<T>::load(__ldcg(p)) : Arith<T>::inf();
+          x[a][e + 1] = i < g.n && j + 1 < g.n ? Arith<T>::load(__ldcg(p + 1)) : Arith<T>::inf();
         }
       }
     const bool late = !mbar_wait_bounded(bar, 0);
-    if (!late) st_product<C, 32, 2, 2, 128, 128, 64, 4>(x, As + 4 * ty, Bs + 4 * tx, g.one);
+    if (!late) st_product<C, 32, 2, 2, 128, 128, 64, 2>(x, As + 4 * ty, Bs + 4 * tx, g.one);
     if (__any_sync(0xffffffffu, late)) {  // give up: wait (bounded) for the copies in flight, store nothing
       if (lane == 0) {
         atomicCAS(g.err, 0, (int)kDevTimeoutTma);
@@ -293,7 +312,7 @@ __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typenam
           const T v1 = last ? Arith<T>::finish(x[a][e + 1]) : (T)x[a][e + 1];
           T *p = g.dst + i * g.dst_ld + j;
           if (pair_out) {
-            *reinterpret_cast<V2 *>(p) = V2{v0, v1};
+            st2(p, v0, v1);
           } else if (i < g.n) {
             if (j < g.n) p[0] = v0;
             if (j + 1 < g.n) p[1] = v1;
@@ -531,7 +550,11 @@ __global__ void __launch_bounds__(kStThreads) __cluster_dims__(kStCluster, 1, 1)
 }
 
 // rest(b) on its own: four CTAs per SM, so that the loads and stores of some
-// run beside the arithmetic of the others.
+// run beside the arithmetic of the others; beside a head CTA two, by shared
+// memory it asks for and does not use (kRestPad): the heads' chain bounds the
+// stage, and with more rest CTAs on its SM a head gets too little of the ALU
+// (n = 1792 int32 590 us with the pad, 667 without).
+constexpr size_t kRestPad = 20 * 1024;
 template <typename T, bool VIA>
 __global__ void __launch_bounds__(kStThreads, 4) fw_rest(const StageArgs<T> g) {
   using C = typename Arith<T>::C;
@@ -554,8 +577,8 @@ __global__ void __launch_bounds__(kStThreads, 4) fw_rest(const StageArgs<T> g) {
 // each head CTA can have an SM to itself, and one launch per stage while rest
 // has a handful of tiles (with more, the next stage's heads are placed two to
 // an SM).  Measured, us per solve: n = 768 int32 164 with W = 32, 173 with 16;
-// n = 512 fp32 104 with 16, 111 with 32; n = 1536 int32 414 with 32, 480 with
-// 64; n = 2048 int32 764 with 64, 902 with 32.  In one launch: n = 256 53 (57
+// n = 512 fp32 104 with 16, 111 with 32; n = 1920 int32 676 with 32, 727 with
+// 64; n = 2048 int32 783 with 64, 822 with 32.  In one launch: n = 256 53 (57
 // with two), n = 512 118 (104), n = 1024 323 (221).
 struct HeadCut {
   int W;        // strip width: 16, 32 or 64
@@ -563,7 +586,7 @@ struct HeadCut {
 };
 inline HeadCut head_cut(int R) {
   if (R <= 9) return {16, R <= 5};
-  if (R <= 24) return {32, false};
+  if (R <= 30) return {32, false};
   return {64, false};
 }
 
@@ -580,6 +603,8 @@ static cudaError_t launch_head(const StageArgs<T> &g, int grid, cudaStream_t st)
         cudaFuncSetAttribute(fw_head<T, W, VIA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fw_head<T, W, VIA>, carve, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fw_rest<T, VIA>, carve, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fw_rest<T, VIA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRestPad);
     if (e != cudaSuccess) return e;
     done |= 1ull << dev;
   }
@@ -623,7 +648,7 @@ static int run_stages(const RunArgs &a) {
       if (e != cudaSuccess) return APSP_ECUDA;
     }
     if (b >= 0 && !merged &&
-        launch(fw_rest<T, VIA>, dim3(g.rest + 1), kStThreads, 0, a.stream, 0, g) != cudaSuccess)
+        launch(fw_rest<T, VIA>, dim3(g.rest + 1), kStThreads, kRestPad, a.stream, 0, g) != cudaSuccess)
       return APSP_ECUDA;
   }
   return cudaPeekAtLastError() == cudaSuccess ? APSP_OK : APSP_ECUDA;

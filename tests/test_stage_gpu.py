@@ -21,6 +21,9 @@ def graph(dt, n, seed):
     if dt == "f32":  # sums are rounded: full 24-bit mantissas
         w = (1.0 - g.random((n, n))).astype(np.float32)
         w[g.random((n, n)) < 0.5] = np.inf
+    elif dt == "i16":  # (n - 1) * 7 < 16383 up to n = 2341
+        w = g.integers(0, 8, (n, n)).astype(np.int16)
+        w[g.random((n, n)) > 0.05] = 16383
     else:
         p = g.integers(0, 51, n)
         w = (g.integers(0, 951, (n, n)) + p[:, None] - p[None, :]).astype(np.int32)
@@ -39,15 +42,17 @@ def on_device(w, ld, offset=0):
     return d
 
 
-@pytest.mark.parametrize("dt", ["f32", "i32"])
+@pytest.mark.parametrize("dt", ["f32", "i32", "i16"])
 @pytest.mark.parametrize("n", [1, 63, 64, 65, 127, 128, 129, 320, 321, 576, 577, 640, 1536, 1537, 1600, 2047, 2048, 2049])
 def test_stage_schedule_equals_plain(dt, n):
     w = graph(dt, n, n)
-    ref = on_device(w, (n + 3) // 4 * 4)
+    ref = on_device(w, (n + 7) // 8 * 8)
     binding.apsp_fw(ref, n, flags=binding.FLAG_NO_LOOKAHEAD | binding.FLAG_NO_GRAPH)
     if dt == "i32" and n <= 1600:
         np.testing.assert_array_equal(ref[:, :n].cpu().numpy(), oracle.fw_int32_conv(w))
-    for ld, offset in ((n, 0), ((n + 3) // 4 * 4, 0), (n + 1, 0), (n + 37, 3)):
+    if dt == "i16" and n <= 1600:
+        np.testing.assert_array_equal(ref[:, :n].cpu().numpy(), oracle.fw_int16_conv(w))
+    for ld, offset in ((n, 0), ((n + 7) // 8 * 8, 0), (n + 1, 0), (n + 37, 3)):
         d = on_device(w, ld, offset)
         binding.apsp_fw(d, n)
         torch.cuda.synchronize()
@@ -56,7 +61,7 @@ def test_stage_schedule_equals_plain(dt, n):
     assert binding.device_error() == 0
 
 
-@pytest.mark.parametrize("dt", ["f32", "i32"])
+@pytest.mark.parametrize("dt", ["f32", "i32", "i16"])
 @pytest.mark.parametrize("n", [64, 65, 200, 321, 577, 1000, 1537])
 def test_stage_schedule_paths(dt, n):
     # the stage record and the distances, against the plain schedule's
