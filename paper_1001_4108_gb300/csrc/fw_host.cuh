@@ -143,16 +143,16 @@ static int run_rounds(const RunArgs &a) {
     if constexpr (HAS_TMA) {
       if (cudaFuncSetAttribute(fw_tile_tma<T, S, 0, VIA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                P3Tma<S>::SMEM) != cudaSuccess ||
+          cudaFuncSetAttribute(fw_tile_tma<T, S, 0, VIA, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               P3Tma<S>::SMEM) != cudaSuccess ||
           cudaFuncSetAttribute(fw_tile_tma<T, S, 1, VIA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                P3Tma<S>::SMEM) != cudaSuccess)
         return APSP_ECUDA;
       if constexpr (std::is_same<T, float>::value) {
         const int sm = P3Tma<S>::SMEM;
         const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        if (cudaFuncSetAttribute(fw_phase3_f32x2<S, false, true, VIA>, attr, sm) != cudaSuccess ||
-            cudaFuncSetAttribute(fw_phase3_f32x2<S, true, true, VIA>, attr, sm) != cudaSuccess ||
-            cudaFuncSetAttribute(fw_phase3_f32x2<S, false, false, VIA>, attr, sm) != cudaSuccess ||
-            cudaFuncSetAttribute(fw_phase3_f32x2<S, true, false, VIA>, attr, sm) != cudaSuccess)
+        if (cudaFuncSetAttribute(fw_phase3_f32x2<S, false, VIA>, attr, sm) != cudaSuccess ||
+            cudaFuncSetAttribute(fw_phase3_f32x2<S, true, VIA>, attr, sm) != cudaSuccess)
           return APSP_ECUDA;
       }
     }
@@ -278,7 +278,7 @@ static int run_rounds(const RunArgs &a) {
                       reinterpret_cast<int16_t *>(d), n, ld, b, R, TileSet{}, reverse, arep[buf_of(b)], a.via,
                       a.via_ld, a.err);
     }
-    T *bpb = (use_packed && full_k(b)) ? bp[buf_of(b)] : nullptr;
+    T *bpb = use_packed ? bp[buf_of(b)] : nullptr;
     if constexpr (HAS_TMA && S == 64 && !std::is_same<T, int16_t>::value) {
       // four strips per panel tile while the stage is latency bound
       if (use_tma && full_k(b) && strips)
@@ -291,8 +291,8 @@ static int run_rounds(const RunArgs &a) {
                       CRoute<T>{d, ld, d, ld}, n, b, R, TileSet{}, last, reverse, bpb, 2 * np, a.via, a.via_ld,
                       a.err);
     }
-    return launch(fw_phase2<T, S, K::NT2>, g, K::NT2, K::SM2, s, prio, d, n, ld, b, R, last, bpb, 2 * np, a.via,
-                  a.via_ld);
+    return launch(fw_phase2<T, S, K::NT2>, g, K::NT2, K::SM2, s, prio, d, n, ld, b, R, last, bpb, 2 * np,
+                  use_s16 ? arep[buf_of(b)] : (uint32_t *)nullptr, a.via, a.via_ld);
   };
   // phase 3 of stage b over the tiles of `kind`
   auto phase3 = [&](int b, int kind, cudaStream_t s, int prio) -> cudaError_t {
@@ -307,53 +307,45 @@ static int run_rounds(const RunArgs &a) {
       cr.dst = static_cast<T *>(a.last_dst);
       cr.dst_ld = a.last_dst_ld;
     }
-    if (full_k(b)) {
-      if constexpr (HAS_TMA && S == 64 && !std::is_same<T, int16_t>::value) {
-        // the cross tiles of the lookahead schedule: as few as the panel
-        // tiles and on the critical path, so cut into strips as well
-        if (kind == kTilesCross && use_tma && strips) {
-          const TileSet ts = make_tileset(kind, kPartAny, b, R, ragged);
-          if (ts.total() == 0) return cudaSuccess;
-          return launch(fw_strip<T, S, 0, VIA>, dim3(4 * ts.total()), 64, 0, s, prio, cr, (const T *)d, n, ld, b,
-                        R, ts, last, reverse, (T *)nullptr, (int64_t)0, a.via, a.via_ld);
-        }
+    // The partial k-block of a ragged last stage runs on the staged kernels too:
+    // phase 2 leaves "infinity" past the matrix in the panel copies (fp32
+    // row panel, int16 column panel), and fw_tile_tma has a form for it.
+    if constexpr (HAS_TMA && S == 64 && !std::is_same<T, int16_t>::value) {
+      // the cross tiles of the lookahead schedule: as few as the panel
+      // tiles and on the critical path, so cut into strips as well
+      if (kind == kTilesCross && use_tma && strips) {
+        const TileSet ts = make_tileset(kind, kPartAny, b, R, ragged);
+        if (ts.total() == 0) return cudaSuccess;
+        return launch(fw_strip<T, S, 0, VIA>, dim3(4 * ts.total()), 64, 0, s, prio, cr, (const T *)d, n, ld, b,
+                      R, ts, last, reverse, (T *)nullptr, (int64_t)0, a.via, a.via_ld);
       }
-      if constexpr (std::is_same<T, int16_t>::value) {
-        if (use_s16) {
-          const TileSet ts = make_tileset(kind, kPartAny, b, R, ragged);
-          if (ts.total() == 0) return cudaSuccess;
-          return launch(fw_tile_s16x2<S, 0, VIA>, dim3(ts.total()), P3S16<S>::TPB, P3S16<S>::SMEM_P3, s, prio,
-                        mArep[buf_of(b)], mB16, mC16, reinterpret_cast<int16_t *>(d), n, ld, b, R, ts, reverse,
-                        arep[buf_of(b)], a.via, a.via_ld, a.err);
-        }
+    }
+    if constexpr (std::is_same<T, int16_t>::value) {
+      if (use_s16) {
+        const TileSet ts = make_tileset(kind, kPartAny, b, R, ragged);
+        if (ts.total() == 0) return cudaSuccess;
+        return launch(fw_tile_s16x2<S, 0, VIA>, dim3(ts.total()), P3S16<S>::TPB, P3S16<S>::SMEM_P3, s, prio,
+                      mArep[buf_of(b)], mB16, mC16, reinterpret_cast<int16_t *>(d), n, ld, b, R, ts, reverse,
+                      arep[buf_of(b)], a.via, a.via_ld, a.err);
       }
-      if constexpr (std::is_same<T, float>::value) {
-        if (use_packed) {
-          const int tpb = P3Tma<S>::TPB, sm = P3Tma<S>::SMEM;
-          const CUtensorMap &mb = mBp[buf_of(b)];
-          const TileSet ti = make_tileset(kind, kPartInterior, b, R, ragged);
-          const TileSet te = make_tileset(kind, kPartEdge, b, R, ragged);
-          cudaError_t e = cudaSuccess;
-          if (ti.total() > 0)
-            e = reverse ? launch(fw_phase3_f32x2<S, true, true, VIA>, dim3(ti.total()), tpb, sm, s, prio, mA, mb,
-                                 cr, n, b, ti, a.via, a.via_ld, a.err)
-                        : launch(fw_phase3_f32x2<S, false, true, VIA>, dim3(ti.total()), tpb, sm, s, prio, mA, mb,
-                                 cr, n, b, ti, a.via, a.via_ld, a.err);
-          if (e == cudaSuccess && te.total() > 0)
-            e = reverse ? launch(fw_phase3_f32x2<S, true, false, VIA>, dim3(te.total()), tpb, sm, s, prio, mA, mb,
-                                 cr, n, b, te, a.via, a.via_ld, a.err)
-                        : launch(fw_phase3_f32x2<S, false, false, VIA>, dim3(te.total()), tpb, sm, s, prio, mA, mb,
-                                 cr, n, b, te, a.via, a.via_ld, a.err);
-          return e;
-        }
+    }
+    if constexpr (std::is_same<T, float>::value) {
+      if (use_packed) {
+        const int tpb = P3Tma<S>::TPB, sm = P3Tma<S>::SMEM;
+        const CUtensorMap &mb = mBp[buf_of(b)];
+        const TileSet ts = make_tileset(kind, kPartAny, b, R, ragged);
+        if (ts.total() == 0) return cudaSuccess;
+        const auto k = reverse ? fw_phase3_f32x2<S, true, VIA> : fw_phase3_f32x2<S, false, VIA>;
+        return launch(k, dim3(ts.total()), tpb, sm, s, prio, mA, mb, cr, n, b, ts, a.via, a.via_ld, a.err);
       }
-      if constexpr (HAS_TMA) {
-        if (use_tma) {
-          const TileSet ts = make_tileset(kind, kPartAny, b, R, ragged);
-          if (ts.total() == 0) return cudaSuccess;
-          return launch(fw_tile_tma<T, S, 0, VIA>, dim3(ts.total()), P3Tma<S>::TPB, P3Tma<S>::SMEM, s, prio, mA, mB, cr,
-                        n, b, R, ts, last, reverse, (T *)nullptr, (int64_t)0, a.via, a.via_ld, a.err);
-        }
+    }
+    if constexpr (HAS_TMA) {
+      if (use_tma) {
+        const TileSet ts = make_tileset(kind, kPartAny, b, R, ragged);
+        if (ts.total() == 0) return cudaSuccess;
+        const auto k = full_k(b) ? fw_tile_tma<T, S, 0, VIA> : fw_tile_tma<T, S, 0, VIA, true>;
+        return launch(k, dim3(ts.total()), P3Tma<S>::TPB, P3Tma<S>::SMEM, s, prio, mA, mB, cr, n, b, R, ts, last,
+                      reverse, (T *)nullptr, (int64_t)0, a.via, a.via_ld, a.err);
       }
     }
     // generic kernel: all tiles of the stage (plain schedule only)

@@ -150,10 +150,14 @@ __global__ void __launch_bounds__((S / 8) * (S / 4), S == 128 ? 2 : 4)
 // into bp: element (k, j) of the pivot row block goes to
 // bp[(k / 2) * bp_ld + 2 * j + (k % 2)] (j = global column, padding included),
 // the layout the packed fp32 phase-3 kernel reads.
+//
+// With arep != nullptr (int16) the column panel tiles are also stored as
+// replicated words, element (i, k) at arep[i * S + k], padding included: what
+// the packed int16x2 phase-3 kernel reads.
 template <typename T, int S, int NT>
 __global__ void __launch_bounds__(NT) fw_phase2(T *__restrict__ d, int64_t n, int64_t ld, int b, int R, int last,
-                                                T *__restrict__ bp, int64_t bp_ld, int16_t *__restrict__ via,
-                                                int64_t via_ld) {
+                                                T *__restrict__ bp, int64_t bp_ld, uint32_t *__restrict__ arep,
+                                                int16_t *__restrict__ via, int64_t via_ld) {
   using C = typename Arith<T>::C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C *D = reinterpret_cast<C *>(smem_raw);
@@ -204,6 +208,12 @@ __global__ void __launch_bounds__(NT) fw_phase2(T *__restrict__ d, int64_t n, in
     for (int r = 0; r < E; ++r) {
       const int i = i0 + RS * r;
       bp[(int64_t)(i >> 1) * bp_ld + 2 * (c0 + j) + (i & 1)] = (T)acc[r];
+    }
+  }
+  if constexpr (std::is_same<T, int16_t>::value) {
+    if (arep && !row_panel) {
+#pragma unroll
+      for (int r = 0; r < E; ++r) arep[(r0 + i0 + RS * r) * S + j] = ((uint32_t)acc[r] & 0xffffu) * 0x10001u;
     }
   }
 }
@@ -357,12 +367,18 @@ __device__ __forceinline__ void lds4(const T *p, T &x0, T &x1, T &x2, T &x3) {
   x3 = *reinterpret_cast<T *>(&e);
 }
 
-template <typename T, int S, int MODE, bool VIA = false>
+// TAIL: the partial k-block of a ragged matrix's last stage.  Its slices past
+// the matrix are not loaded, and the rows of B past it, which TMA fills with
+// zeros, are overwritten with "infinity" in shared memory (so what A holds
+// there does not matter).
+template <typename T, int S, int MODE, bool VIA = false, bool TAIL = false>
 __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
     fw_tile_tma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const CRoute<T> cr, int64_t n, int b, int R, const TileSet ts, int last, int reverse,
                 T *__restrict__ bp, int64_t bp_ld, int16_t *__restrict__ via, int64_t via_ld, int *err) {
   using P = P3Tma<S>;
+  const int kvalid = TAIL ? (int)(n - (int64_t)b * S) : S;
+  const int nsl = TAIL ? (kvalid + P::KS - 1) / P::KS : P::NSL;
   constexpr int G = P::G;
   constexpr int KS = P::KS;
   extern __shared__ unsigned char smem_raw[];
@@ -394,7 +410,7 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
 #pragma unroll
     for (int s = 0; s < P::STAGES; ++s) mbar_init(&full[s], 1);
     fence_mbar_init();
-    ring_ctl_init(ring, P::STAGES < P::NSL ? P::STAGES : P::NSL);
+    ring_ctl_init(ring, P::STAGES < nsl ? P::STAGES : nsl);
     tile_ij[0] = It;
     tile_ij[1] = Jt;
   }
@@ -402,7 +418,7 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
   wait_prior_grid();
   if (tid == 0) {
 #pragma unroll
-    for (int s = 0; s < P::STAGES && s < P::NSL; ++s) {
+    for (int s = 0; s < P::STAGES && s < nsl; ++s) {
       mbar_arrive_expect_tx(&full[s], P::A_BYTES + P::B_BYTES);
       tma_load_2d(As + s * (S * KS), &tmA, &full[s], k0 + s * KS, (int)I0);
       tma_load_2d(Bs + s * (KS * S), &tmB, &full[s], (int)J0, k0 + s * KS);
@@ -432,9 +448,15 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
 
   bool timed_out = false;
   const int sw = ty & 7;  // swizzle phase of every row this thread reads
-  for (int s = 0; s < P::NSL; ++s) {
+  for (int s = 0; s < nsl; ++s) {
     const int st = s % P::STAGES;
     if (!timed_out && !mbar_wait_bounded(&full[st], (s / P::STAGES) & 1)) timed_out = true;
+    if constexpr (TAIL) {
+      if ((s + 1) * KS > kvalid) {
+        for (int e = (kvalid - s * KS) * S + tid; e < KS * S; e += P::TPB) Bs[st * (KS * S) + e] = Arith<T>::inf();
+        __syncthreads();
+      }
+    }
     const T *A = As + st * (S * KS) + ty * KS;
     const T *B = Bs + st * (KS * S) + 4 * tx;
     if constexpr (std::is_same<T, float>::value) {
@@ -486,7 +508,7 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
     }
     // the last warp done with stage st refills it with slice s + STAGES (no
     // CTA barrier per slice)
-    if (s + P::STAGES < P::NSL)
+    if (s + P::STAGES < nsl)
       ring_release<P::STAGES, P::TPB / 32>(ring, st, timed_out, [&] {
         const int s2 = s + P::STAGES;
         mbar_arrive_expect_tx(&full[st], P::A_BYTES + P::B_BYTES);
@@ -563,10 +585,13 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
 // load yields the (k, k+1) pairs of two adjacent columns.  Thread columns:
 // j = 2 (tx + G m) + e, m < 4, e < 2.
 //
-// blockIdx.x numbers the tiles of the launch's tile set.  FULL = true: every
-// row and column of every tile is inside the matrix (interior tiles); FULL =
-// false: masked loads/stores (the edge tiles of a ragged matrix).
-template <int S, bool REVERSE, bool FULL, bool VIA = false>
+// blockIdx.x numbers the tiles of the launch's tile set.  Each CTA looks whether
+// its tile is inside the matrix; the edge tiles of a ragged one are loaded and
+// stored with masks.  (As launches of their own the edge tiles were a fraction
+// of a wave, about 11 us per stage: fp32 n = 6000 12.98 ms against 12.28.  A
+// form without the masks for interior tiles is no faster: n = 16384 231.6 ms
+// against 227.8, n = 4096 4.71 against 4.24; ptxas then spills more.)
+template <int S, bool REVERSE, bool VIA = false>
 __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
     fw_phase3_f32x2(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBp,
                     const CRoute<float> cr, int64_t n, int b, const TileSet ts, int16_t *__restrict__ via,
@@ -615,26 +640,27 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
   uint64_t cbase =
       reinterpret_cast<uint64_t>(cr.src + ((int64_t)It * S + ty) * cr.src_ld + (int64_t)Jt * S + 2 * tx);
   int64_t rstride = (int64_t)G * cr.src_ld * (int64_t)sizeof(float);
-  int rows_left = 0, cols_left = 0;  // (masked form) rows/cols of the tile inside the matrix, from this thread
-  if (!FULL) {
-    rows_left = (int)(n - ((int64_t)It * S + ty));
-    cols_left = (int)(n - ((int64_t)Jt * S + 2 * tx));
-  }
+  if ((int64_t)(It + 1) * S <= n && (int64_t)(Jt + 1) * S <= n) {
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const float *pc = reinterpret_cast<const float *>(cbase + r * rstride + 8 * G * m);
-      if (FULL) {
-        const float2 v = *reinterpret_cast<const float2 *>(pc);
+      for (int m = 0; m < 4; ++m) {
+        const float2 v = *reinterpret_cast<const float2 *>(cbase + r * rstride + 8 * G * m);
         acc[r][2 * m] = v.x;
         acc[r][2 * m + 1] = v.y;
-      } else {
+      }
+  } else {  // rows and columns of the tile inside the matrix, from this thread's on
+    const int rows_left = (int)(n - ((int64_t)It * S + ty)), cols_left = (int)(n - ((int64_t)Jt * S + 2 * tx));
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const float *pc = reinterpret_cast<const float *>(cbase + r * rstride + 8 * G * m);
         const bool rok = G * r < rows_left;
         acc[r][2 * m] = (rok && 2 * G * m < cols_left) ? pc[0] : Arith<float>::inf();
         acc[r][2 * m + 1] = (rok && 2 * G * m + 1 < cols_left) ? pc[1] : Arith<float>::inf();
       }
-    }
+  }
 
   bool timed_out = false;
   const int sw = ty & 7;
@@ -696,10 +722,6 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
   asm volatile("" : "+r"(It2), "+r"(Jt2), "+r"(ty2), "+r"(tx2));
   cbase = reinterpret_cast<uint64_t>(cr.dst + ((int64_t)It2 * S + ty2) * cr.dst_ld + (int64_t)Jt2 * S + 2 * tx2);
   rstride = (int64_t)G * cr.dst_ld * (int64_t)sizeof(float);
-  if (!FULL) {
-    rows_left = (int)(n - ((int64_t)It2 * S + ty2));
-    cols_left = (int)(n - ((int64_t)Jt2 * S + 2 * tx2));
-  }
   if (VIA && via) {  // path bookkeeping: compare with the values about to be replaced
 #pragma unroll
     for (int r = 0; r < 8; ++r)
@@ -711,19 +733,24 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
           if (gi < n && gj < n) note_via(via, via_ld, gi, gj, acc[r][2 * m + e], cr.src[gi * cr.src_ld + gj], b);
         }
   }
+  if ((int64_t)(It2 + 1) * S <= n && (int64_t)(Jt2 + 1) * S <= n) {
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      float *pc = reinterpret_cast<float *>(cbase + r * rstride + 8 * G * m);
-      if (FULL) {
-        *reinterpret_cast<float2 *>(pc) = make_float2(acc[r][2 * m], acc[r][2 * m + 1]);
-      } else {
+      for (int m = 0; m < 4; ++m)
+        *reinterpret_cast<float2 *>(cbase + r * rstride + 8 * G * m) = make_float2(acc[r][2 * m], acc[r][2 * m + 1]);
+  } else {
+    const int rows_left = (int)(n - ((int64_t)It2 * S + ty2)), cols_left = (int)(n - ((int64_t)Jt2 * S + 2 * tx2));
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        float *pc = reinterpret_cast<float *>(cbase + r * rstride + 8 * G * m);
         const bool rok = G * r < rows_left;
         if (rok && 2 * G * m < cols_left) pc[0] = acc[r][2 * m];
         if (rok && 2 * G * m + 1 < cols_left) pc[1] = acc[r][2 * m + 1];
       }
-    }
+  }
 }
 
 // ------------------------------------------- strips (latency-bound launches)
