@@ -463,9 +463,15 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   const int R = (int)((n + a.S - 1) / a.S);
   const size_t stage_need =
       uses_stage_launches(a.S, R, dtype == APSP_I16, a.flags, a.events != nullptr) ? stage_ws_bytes(R) : 0;
-  if (need || stage_need) {
+  // the int32 kernels that read both panels from copies, not the matrix
+  constexpr int kNoPairs = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_WORKSPACE;
+  const size_t pairs_need = stage_need || dtype != APSP_I32 || R < 2 || (a.flags & kNoPairs)
+                                ? 0
+                                : (R >= kLookaheadMinRounds ? 4 : 2) * interleaved_panel_bytes(n, a.S);
+  const size_t more = std::max(stage_need, pairs_need);
+  if (need || more) {
     if (opt && opt->workspace && !need) {
-      // not asked for: taken if it serves the one-launch-per-stage schedule
+      // not asked for: taken if it is enough for the kernels that can use one
       a.ws = opt->workspace;
       a.ws_bytes = (size_t)std::max<int64_t>(opt->workspace_bytes, 0);
     } else if (opt && opt->workspace) {
@@ -476,7 +482,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       a.ws = opt->workspace;
       a.ws_bytes = (size_t)opt->workspace_bytes;
     } else {
-      a.ws = library_workspace(dev, a.stream, std::max(need, stage_need), cap != cudaStreamCaptureStatusNone,
+      a.ws = library_workspace(dev, a.stream, std::max(need, more), cap != cudaStreamCaptureStatusNone,
                                &a.ws_bytes);
       if (!a.ws) a.ws_bytes = 0;  // the kernels fall back to the form that needs none
     }

@@ -76,7 +76,7 @@ static bool make_panel_maps(T *d, int64_t n, int64_t ld, CUtensorMap *mA, CUtens
 
 // Tensor map of the k-pair interleaved row panel (S/2 rows x 2 n_p floats).
 template <int S>
-static bool make_interleaved_map(float *bp, int64_t np, CUtensorMap *m) {
+static bool make_interleaved_map(void *bp, int64_t np, CUtensorMap *m) {
   EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)(2 * np), (cuuint64_t)(S / 2)};
@@ -148,6 +148,11 @@ static int run_rounds(const RunArgs &a) {
           cudaFuncSetAttribute(fw_tile_tma<T, S, 1, VIA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                P3Tma<S>::SMEM) != cudaSuccess)
         return APSP_ECUDA;
+      if constexpr (std::is_same<T, int32_t>::value) {
+        if (cudaFuncSetAttribute(fw_phase3_pairs<S, VIA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 P3Tma<S>::SMEM) != cudaSuccess)
+          return APSP_ECUDA;
+      }
       if constexpr (std::is_same<T, float>::value) {
         const int sm = P3Tma<S>::SMEM;
         const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
@@ -193,22 +198,41 @@ static int run_rounds(const RunArgs &a) {
 
   // Tensor maps; the panel copies of phase 2 (one buffer, or two for the
   // lookahead schedule).
-  CUtensorMap mA, mB, mBp[2];
-  bool use_tma = false, use_packed = false;
-  T *bp[2] = {nullptr, nullptr};
+  CUtensorMap mA, mB, mBp[2], mAp[2];
+  bool use_tma = false, use_packed = false, use_pairs = false;
+  T *bp[2] = {nullptr, nullptr}, *ap[2] = {nullptr, nullptr};
   int nbuf = 0;
   if constexpr (HAS_TMA) {
     use_tma = a.tma_ok && !generic_only && R > 1 && make_panel_maps<T, S>(d, n, ld, &mA, &mB);
+    const size_t pb = interleaved_panel_bytes(n, S);
+    const bool ws_ok = use_tma && a.ws && reinterpret_cast<uintptr_t>(a.ws) % 256 == 0;
+    if constexpr (std::is_same<T, int32_t>::value) {
+      // both panels: one buffer each, two for the lookahead schedule
+      const int nb = R >= kLookaheadMinRounds ? 2 : 1;
+      if (ws_ok && !reverse && a.ws_bytes >= 2 * nb * pb) {
+        use_pairs = true;
+        for (int i = 0; i < nb; ++i) {
+          bp[i] = reinterpret_cast<T *>(static_cast<char *>(a.ws) + 2 * i * pb);
+          ap[i] = reinterpret_cast<T *>(static_cast<char *>(a.ws) + (2 * i + 1) * pb);
+          use_pairs = use_pairs && make_interleaved_map<S>(bp[i], np, &mBp[i]) &&
+                      make_interleaved_map<S>(ap[i], np, &mAp[i]);
+        }
+        if (use_pairs) nbuf = nb;
+        else bp[0] = bp[1] = ap[0] = ap[1] = nullptr;
+      }
+    }
     if constexpr (std::is_same<T, float>::value) {
-      const size_t pb = interleaved_panel_bytes(n, S);
-      if (use_tma && a.ws && a.ws_bytes >= pb && reinterpret_cast<uintptr_t>(a.ws) % 256 == 0) {
+      if (ws_ok && a.ws_bytes >= pb) {
         nbuf = a.ws_bytes >= 2 * pb ? 2 : 1;
         use_packed = true;
         for (int i = 0; i < nbuf; ++i) {
           bp[i] = reinterpret_cast<T *>(static_cast<char *>(a.ws) + i * pb);
-          use_packed = use_packed && make_interleaved_map<S>(reinterpret_cast<float *>(bp[i]), np, &mBp[i]);
+          use_packed = use_packed && make_interleaved_map<S>(bp[i], np, &mBp[i]);
         }
-        if (!use_packed) nbuf = 0;
+        if (!use_packed) {
+          nbuf = 0;
+          bp[0] = bp[1] = nullptr;
+        }
       }
     }
   }
@@ -235,7 +259,7 @@ static int run_rounds(const RunArgs &a) {
   bool p3_tma = false;
   if constexpr (std::is_same<T, int16_t>::value) p3_tma = use_s16;
   else p3_tma = use_tma;
-  const bool needs_panel = use_packed || use_s16;
+  const bool needs_panel = use_packed || use_pairs || use_s16;
   // A caller that supplies its workspace for the packed fp32 kernels (the
   // allocation-free entry point) is told when they cannot run on it, before
   // any work is enqueued, instead of getting the unpacked kernels silently.
@@ -278,20 +302,20 @@ static int run_rounds(const RunArgs &a) {
                       reinterpret_cast<int16_t *>(d), n, ld, b, R, TileSet{}, reverse, arep[buf_of(b)], a.via,
                       a.via_ld, a.err);
     }
-    T *bpb = use_packed ? bp[buf_of(b)] : nullptr;
+    T *bpb = bp[buf_of(b)], *apb = ap[buf_of(b)];
     if constexpr (HAS_TMA && S == 64 && !std::is_same<T, int16_t>::value) {
       // four strips per panel tile while the stage is latency bound
       if (use_tma && full_k(b) && strips)
         return launch(fw_strip<T, S, 1, VIA>, dim3(8 * (R - 1)), 64, 0, s, prio, CRoute<T>{d, ld, d, ld},
-                      (const T *)d, n, ld, b, R, TileSet{}, last, reverse, bpb, 2 * np, a.via, a.via_ld);
+                      (const T *)d, n, ld, b, R, TileSet{}, last, reverse, bpb, apb, 2 * np, a.via, a.via_ld);
     }
     if constexpr (HAS_TMA) {
       if (use_tma && full_k(b))
         return launch(fw_tile_tma<T, S, 1, VIA>, g, P3Tma<S>::TPB, P3Tma<S>::SMEM, s, prio, mA, mB,
-                      CRoute<T>{d, ld, d, ld}, n, b, R, TileSet{}, last, reverse, bpb, 2 * np, a.via, a.via_ld,
-                      a.err);
+                      CRoute<T>{d, ld, d, ld}, n, b, R, TileSet{}, last, reverse, bpb, apb, 2 * np, a.via,
+                      a.via_ld, a.err);
     }
-    return launch(fw_phase2<T, S, K::NT2>, g, K::NT2, K::SM2, s, prio, d, n, ld, b, R, last, bpb, 2 * np,
+    return launch(fw_phase2<T, S, K::NT2>, g, K::NT2, K::SM2, s, prio, d, n, ld, b, R, last, bpb, apb, 2 * np,
                   use_s16 ? arep[buf_of(b)] : (uint32_t *)nullptr, a.via, a.via_ld);
   };
   // phase 3 of stage b over the tiles of `kind`
@@ -317,7 +341,15 @@ static int run_rounds(const RunArgs &a) {
         const TileSet ts = make_tileset(kind, kPartAny, b, R, ragged);
         if (ts.total() == 0) return cudaSuccess;
         return launch(fw_strip<T, S, 0, VIA>, dim3(4 * ts.total()), 64, 0, s, prio, cr, (const T *)d, n, ld, b,
-                      R, ts, last, reverse, (T *)nullptr, (int64_t)0, a.via, a.via_ld);
+                      R, ts, last, reverse, (T *)nullptr, (T *)nullptr, (int64_t)0, a.via, a.via_ld);
+      }
+    }
+    if constexpr (std::is_same<T, int32_t>::value) {
+      if (use_pairs) {
+        const TileSet ts = make_tileset(kind, kPartAny, b, R, ragged);
+        if (ts.total() == 0) return cudaSuccess;
+        return launch(fw_phase3_pairs<S, VIA>, dim3(ts.total()), P3Tma<S>::TPB, P3Tma<S>::SMEM, s, prio,
+                      mAp[buf_of(b)], mBp[buf_of(b)], cr, n, b, ts, last, 1, a.via, a.via_ld, a.err);
       }
     }
     if constexpr (std::is_same<T, int16_t>::value) {
@@ -345,7 +377,7 @@ static int run_rounds(const RunArgs &a) {
         if (ts.total() == 0) return cudaSuccess;
         const auto k = full_k(b) ? fw_tile_tma<T, S, 0, VIA> : fw_tile_tma<T, S, 0, VIA, true>;
         return launch(k, dim3(ts.total()), P3Tma<S>::TPB, P3Tma<S>::SMEM, s, prio, mA, mB, cr, n, b, R, ts, last,
-                      reverse, (T *)nullptr, (int64_t)0, a.via, a.via_ld, a.err);
+                      reverse, (T *)nullptr, (T *)nullptr, (int64_t)0, a.via, a.via_ld, a.err);
       }
     }
     // generic kernel: all tiles of the stage (plain schedule only)

@@ -150,14 +150,17 @@ __global__ void __launch_bounds__((S / 8) * (S / 4), S == 128 ? 2 : 4)
 // into bp: element (k, j) of the pivot row block goes to
 // bp[(k / 2) * bp_ld + 2 * j + (k % 2)] (j = global column, padding included),
 // the layout the packed fp32 phase-3 kernel reads.
+// With ap != nullptr the column panel tiles go to ap the same way, rows and
+// columns exchanged: element (i, k) at ap[(k / 2) * bp_ld + 2 * i + (k % 2)].
 //
 // With arep != nullptr (int16) the column panel tiles are also stored as
 // replicated words, element (i, k) at arep[i * S + k], padding included: what
 // the packed int16x2 phase-3 kernel reads.
 template <typename T, int S, int NT>
 __global__ void __launch_bounds__(NT) fw_phase2(T *__restrict__ d, int64_t n, int64_t ld, int b, int R, int last,
-                                                T *__restrict__ bp, int64_t bp_ld, uint32_t *__restrict__ arep,
-                                                int16_t *__restrict__ via, int64_t via_ld) {
+                                                T *__restrict__ bp, T *__restrict__ ap, int64_t bp_ld,
+                                                uint32_t *__restrict__ arep, int16_t *__restrict__ via,
+                                                int64_t via_ld) {
   using C = typename Arith<T>::C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C *D = reinterpret_cast<C *>(smem_raw);
@@ -209,6 +212,11 @@ __global__ void __launch_bounds__(NT) fw_phase2(T *__restrict__ d, int64_t n, in
       const int i = i0 + RS * r;
       bp[(int64_t)(i >> 1) * bp_ld + 2 * (c0 + j) + (i & 1)] = (T)acc[r];
     }
+  }
+  if (ap && !row_panel) {
+#pragma unroll
+    for (int r = 0; r < E; ++r)
+      ap[(int64_t)(j >> 1) * bp_ld + 2 * (r0 + i0 + RS * r) + (j & 1)] = (T)acc[r];
   }
   if constexpr (std::is_same<T, int16_t>::value) {
     if (arep && !row_panel) {
@@ -310,10 +318,11 @@ __global__ void __launch_bounds__(256) fw_phase3_generic(T *__restrict__ d, int6
 // The C tile goes global -> registers with 128-bit loads issued before the
 // first wait, so they overlap the first TMA copies.
 //
-// With bp != nullptr (phase 2, fp32) the row panel tiles are also written,
-// k-pair interleaved, to bp: element (k, j) of the pivot row block goes to
+// With bp != nullptr (phase 2) the row panel tiles are also written, k-pair
+// interleaved, to bp: element (k, j) of the pivot row block goes to
 // bp[(k / 2) * bp_ld + 2 * j + (k % 2)] (j = global column, padding
-// included), the layout the packed fp32 phase-3 kernel reads.
+// included); with ap != nullptr the column panel tiles, element (i, k) to
+// ap[(k / 2) * bp_ld + 2 * i + (k % 2)].  The phase-3 kernels read these.
 template <int S> struct P3Tma {
   static constexpr int G = S / 8;
   static constexpr int TPB = G * G;
@@ -339,6 +348,15 @@ __device__ __forceinline__ void ld4<float>(const float *p, float &x0, float &x1,
   x0 = v.x; x1 = v.y; x2 = v.z; x3 = v.w;
 }
 template <typename T>
+struct Vec4;
+template <> struct Vec4<float> { using V = float4; };
+template <> struct Vec4<int32_t> { using V = int4; };
+__device__ __forceinline__ void ld2(const int32_t *p, int32_t &x, int32_t &y) {
+  const int2 v = *reinterpret_cast<const int2 *>(p);
+  x = v.x;
+  y = v.y;
+}
+template <typename T>
 __device__ __forceinline__ void st4(T *p, T x0, T x1, T x2, T x3);
 template <>
 __device__ __forceinline__ void st4<int32_t>(int32_t *p, int32_t x0, int32_t x1, int32_t x2, int32_t x3) {
@@ -347,6 +365,11 @@ __device__ __forceinline__ void st4<int32_t>(int32_t *p, int32_t x0, int32_t x1,
 template <>
 __device__ __forceinline__ void st4<float>(float *p, float x0, float x1, float x2, float x3) {
   *reinterpret_cast<float4 *>(p) = make_float4(x0, x1, x2, x3);
+}
+__device__ __forceinline__ void st2(float *p, float x, float y) { *reinterpret_cast<float2 *>(p) = make_float2(x, y); }
+__device__ __forceinline__ void st2(int32_t *p, int32_t x, int32_t y) { *reinterpret_cast<int2 *>(p) = make_int2(x, y); }
+__device__ __forceinline__ void st2(int16_t *p, int16_t x, int16_t y) {
+  *reinterpret_cast<short2 *>(p) = make_short2(x, y);
 }
 // Shared-memory loads the compiler may not merge or hoist across the k-pair
 // loop (keeps the 64 accumulators within two CTAs per SM worth of registers).
@@ -375,7 +398,8 @@ template <typename T, int S, int MODE, bool VIA = false, bool TAIL = false>
 __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
     fw_tile_tma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const CRoute<T> cr, int64_t n, int b, int R, const TileSet ts, int last, int reverse,
-                T *__restrict__ bp, int64_t bp_ld, int16_t *__restrict__ via, int64_t via_ld, int *err) {
+                T *__restrict__ bp, T *__restrict__ ap, int64_t bp_ld, int16_t *__restrict__ via, int64_t via_ld,
+                int *err) {
   using P = P3Tma<S>;
   const int kvalid = TAIL ? (int)(n - (int64_t)b * S) : S;
   const int nsl = TAIL ? (kvalid + P::KS - 1) / P::KS : P::NSL;
@@ -571,6 +595,15 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
       }
     }
   }
+  if (MODE == 1 && ap && !row_panel) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int c = 0; c < 8; c += 2) {
+        const int k = (c / 4) * (S / 2) + 4 * tx + (c % 4);
+        st2(ap + (int64_t)(k >> 1) * bp_ld + 2 * (I0 + ty + G * r), acc[r][c], acc[r][c + 1]);
+      }
+  }
 }
 
 // ------------------------------------------- phase 3, fp32 packed form
@@ -753,6 +786,157 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
   }
 }
 
+// -------------------------------------- phase 3, int32, k-pair interleaved
+// Same tiling and TMA ring, with both operands from the panel copies of phase
+// 2 (ap, bp): a slice is 16 k-pairs x 2S words of each, and one 128-bit load
+// yields (k, k + 1) of two adjacent rows or columns.  With two k's at hand,
+// part of the sums can be formed on the FMA pipe and folded by a three-input
+// min (relax2), which takes half an ALU slot per relaxation; with DPX alone
+// (fw_tile_tma) the ALU pipe is the bound at 64 per clock and SM.  How many,
+// and the unrolling, by measurement (n = 16384: half of them and 8 226.4 ms,
+// half and 4 229.6, 3/8 and 8 232.4, 1/4 and 4 285; n = 4032, s = 64: 3/8 and
+// 4 3.98 ms, half and 4 4.12, 3/8 and 8 4.10).  Volatile loads: plain ones are
+// hoisted and spill (245 ms).  Against fw_tile_tma: n = 16384 235.7 -> 226.4
+// ms, n = 4032 4.33 -> 3.98.  The fp32 kernel gains nothing from this layout
+// (n = 8192 30.3 ms against 29.2).
+// Thread rows: 2 (ty + G m) + e, columns 2 (tx + G m) + e, m < 4, e < 2.
+template <int S, bool VIA>
+__global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
+    fw_phase3_pairs(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                    const CRoute<int32_t> cr, int64_t n, int b, const TileSet ts, int last, int one,
+                    int16_t *__restrict__ via, int64_t via_ld, int *err) {
+  using P = P3Tma<S>;
+  using T = int32_t;
+  constexpr int G = P::G;
+  constexpr int KS = P::KS;
+  constexpr int KP = KS / 2;  // k-pairs per slice
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char *base =
+      reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  T *As = reinterpret_cast<T *>(base);
+  T *Bs = reinterpret_cast<T *>(base + P::STAGES * P::A_BYTES);
+  uint64_t *full = reinterpret_cast<uint64_t *>(base + P::STAGES * (P::A_BYTES + P::B_BYTES));
+  RingCtl<P::STAGES> *ring = reinterpret_cast<RingCtl<P::STAGES> *>(full + P::STAGES);
+
+  const int tid = threadIdx.x;
+  const int tx = tid % G, ty = tid / G;
+  int It, Jt;
+  ts.tile(blockIdx.x, It, Jt);
+
+  if (tid == 0) {
+    prefetch_tensormap(&tmA);
+    prefetch_tensormap(&tmB);
+#pragma unroll
+    for (int s = 0; s < P::STAGES; ++s) mbar_init(&full[s], 1);
+    fence_mbar_init();
+    ring_ctl_init(ring, P::STAGES < P::NSL ? P::STAGES : P::NSL);
+  }
+  __syncthreads();
+  wait_prior_grid();
+  if (tid == 0) {
+#pragma unroll
+    for (int s = 0; s < P::STAGES && s < P::NSL; ++s) {
+      mbar_arrive_expect_tx(&full[s], P::A_BYTES + P::B_BYTES);
+      tma_load_2d(As + s * (S * KS), &tmA, &full[s], 2 * It * S, s * KP);
+      tma_load_2d(Bs + s * (KS * S), &tmB, &full[s], 2 * Jt * S, s * KP);
+    }
+  }
+
+  // C tile -> registers; the addresses again after the main loop, from copies
+  // the compiler cannot see through
+  T acc[8][8];
+  {
+    const T *p = cr.src + ((int64_t)It * S + 2 * ty) * cr.src_ld + (int64_t)Jt * S + 2 * tx;
+    const bool whole = (int64_t)(It + 1) * S <= n && (int64_t)(Jt + 1) * S <= n;
+    const int rows_left = (int)(n - ((int64_t)It * S + 2 * ty)), cols_left = (int)(n - ((int64_t)Jt * S + 2 * tx));
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int i = 2 * G * (r / 2) + r % 2, j = 2 * G * m;
+        const T *q = p + i * cr.src_ld + j;
+        if (whole) {
+          ld2(q, acc[r][2 * m], acc[r][2 * m + 1]);
+        } else {
+          acc[r][2 * m] = (i < rows_left && j < cols_left) ? q[0] : Arith<T>::inf();
+          acc[r][2 * m + 1] = (i < rows_left && j + 1 < cols_left) ? q[1] : Arith<T>::inf();
+        }
+      }
+  }
+
+  bool timed_out = false;
+  for (int s = 0; s < P::NSL; ++s) {
+    const int st = s % P::STAGES;
+    if (!timed_out && !mbar_wait_bounded(&full[st], (s / P::STAGES) & 1)) timed_out = true;
+    const T *A = As + st * (S * KS) + 4 * ty;
+    const T *B = Bs + st * (KS * S) + 4 * tx;
+#pragma unroll(S == 128 ? 8 : 4)
+    for (int p = 0; p < KP; ++p) {
+      int4 av[4], bv[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) lds4<T>(A + p * (2 * S) + 4 * G * m, av[m].x, av[m].y, av[m].z, av[m].w);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) lds4<T>(B + p * (2 * S) + 4 * G * m, bv[m].x, bv[m].y, bv[m].z, bv[m].w);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const T a0 = r % 2 ? av[r / 2].z : av[r / 2].x, a1 = r % 2 ? av[r / 2].w : av[r / 2].y;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          if (r % 2) {
+            acc[r][2 * m] = relax2<false>(acc[r][2 * m], a0, a1, bv[m].x, bv[m].y, one);
+            acc[r][2 * m + 1] = S == 128 || m % 2 ? relax2<true>(acc[r][2 * m + 1], a0, a1, bv[m].z, bv[m].w, one)
+                                                  : relax2<false>(acc[r][2 * m + 1], a0, a1, bv[m].z, bv[m].w, one);
+          } else {
+            acc[r][2 * m] = relax2<true>(acc[r][2 * m], a0, a1, bv[m].x, bv[m].y, one);
+            acc[r][2 * m + 1] = relax2<false>(acc[r][2 * m + 1], a0, a1, bv[m].z, bv[m].w, one);
+          }
+        }
+      }
+    }
+    // the last warp done with stage st refills it with slice s + STAGES
+    if (s + P::STAGES < P::NSL)
+      ring_release<P::STAGES, P::TPB / 32>(ring, st, timed_out, [&] {
+        const int s2 = s + P::STAGES;
+        mbar_arrive_expect_tx(&full[st], P::A_BYTES + P::B_BYTES);
+        tma_load_2d(As + st * (S * KS), &tmA, &full[st], 2 * It * S, s2 * KP);
+        tma_load_2d(Bs + st * (KS * S), &tmB, &full[st], 2 * Jt * S, s2 * KP);
+      });
+  }
+  if (__any_sync(0xffffffffu, timed_out)) {
+    if ((tid & 31) == 0) ring_drain(ring, full, err);
+    return;
+  }
+
+  int It2 = It, Jt2 = Jt, ty2 = ty, tx2 = tx;
+  asm volatile("" : "+r"(It2), "+r"(Jt2), "+r"(ty2), "+r"(tx2));
+  const int64_t i0 = (int64_t)It2 * S + 2 * ty2, j0 = (int64_t)Jt2 * S + 2 * tx2;
+  const bool whole = (int64_t)(It2 + 1) * S <= n && (int64_t)(Jt2 + 1) * S <= n;
+  if (VIA && via) {  // path bookkeeping: compare with the values about to be replaced
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const int64_t gi = i0 + 2 * G * (r / 2) + r % 2, gj = j0 + 2 * G * (c / 2) + c % 2;
+        if (gi < n && gj < n) note_via(via, via_ld, gi, gj, acc[r][c], cr.src[gi * cr.src_ld + gj], b);
+      }
+  }
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int64_t i = i0 + 2 * G * (r / 2) + r % 2, j = j0 + 2 * G * m;
+      T *q = cr.dst + i * cr.dst_ld + j;
+      const T v0 = last ? Arith<T>::finish(acc[r][2 * m]) : acc[r][2 * m];
+      const T v1 = last ? Arith<T>::finish(acc[r][2 * m + 1]) : acc[r][2 * m + 1];
+      if (whole) {
+        st2(q, v0, v1);
+      } else if (i < n) {
+        if (j < n) q[0] = v0;
+        if (j + 1 < n) q[1] = v1;
+      }
+    }
+}
+
 // ------------------------------------------- strips (latency-bound launches)
 // With s = 64 the panel launch of a stage has 2(R-1) tiles and the cross
 // launch of the lookahead schedule about as many; for small n that is fewer
@@ -775,11 +959,6 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
 // Thread (tr, tc) of a RS x CS strip owns rows 4tr..4tr+3 and columns
 // 4tc..4tc+3; per k it reads four A values (shared memory keeps A transposed,
 // AT[k][r]) and four B values, each as one 128-bit load.
-template <typename T>
-struct Vec4;
-template <> struct Vec4<float> { using V = float4; };
-template <> struct Vec4<int32_t> { using V = int4; };
-
 // Elements j..j+3 of a row (j % 4 == 0), "infinity" from column n on; columns
 // n..ld-1 are not read.
 template <typename T>
@@ -793,7 +972,8 @@ __device__ __forceinline__ typename Vec4<T>::V load_row4(const T *row, int64_t j
 template <typename T, int S, int RS, int CS, bool VIA>
 __device__ __forceinline__ void strip_body(const CRoute<T> &cr, const T *__restrict__ d, int64_t n, int64_t ld, int b,
                                            int64_t I0, int64_t J0, int last, int reverse, T *__restrict__ bp,
-                                           int64_t bp_ld, int16_t *__restrict__ via, int64_t via_ld, T *sm) {
+                                           T *__restrict__ ap, int64_t bp_ld, int16_t *__restrict__ via,
+                                           int64_t via_ld, T *sm) {
   using V = typename Vec4<T>::V;
   T *AT = sm;            // [S][RS]
   T *Bs = sm + S * RS;   // [S][CS]
@@ -868,6 +1048,13 @@ __device__ __forceinline__ void strip_body(const CRoute<T> &cr, const T *__restr
         p[1] = acc[a + 1][c];
       }
   }
+  if (ap) {  // and the column panel (the strip holds all of the k-block's columns)
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int c = 0; c < 4; c += 2)
+        st2(ap + (int64_t)((4 * tc + c) >> 1) * bp_ld + 2 * (gi0 + a), acc[a][c], acc[a][c + 1]);
+  }
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
     const int64_t gi = gi0 + a;
@@ -896,8 +1083,8 @@ __device__ __forceinline__ void strip_body(const CRoute<T> &cr, const T *__restr
 template <typename T, int S, int MODE, bool VIA = false>
 __global__ void __launch_bounds__(64) fw_strip(const CRoute<T> cr, const T *__restrict__ d, int64_t n, int64_t ld,
                                                int b, int R, const TileSet ts, int last, int reverse,
-                                               T *__restrict__ bp, int64_t bp_ld, int16_t *__restrict__ via,
-                                               int64_t via_ld) {
+                                               T *__restrict__ bp, T *__restrict__ ap, int64_t bp_ld,
+                                               int16_t *__restrict__ via, int64_t via_ld) {
   static_assert(S == 64, "strips are cut from 64 x 64 tiles");
   __shared__ __align__(16) T sm[S * (S + S / 4)];  // A and B of one strip
   const int t = blockIdx.x / 4, q = blockIdx.x % 4;
@@ -912,11 +1099,11 @@ __global__ void __launch_bounds__(64) fw_strip(const CRoute<T> cr, const T *__re
   wait_prior_grid();
   const int64_t I0 = (int64_t)It * S, J0 = (int64_t)Jt * S;
   if (MODE == 1 && Jt == b)  // column panel: row strips
-    strip_body<T, S, S / 4, S, VIA>(cr, d, n, ld, b, I0 + q * (S / 4), J0, last, reverse, nullptr, 0, via, via_ld,
-                                    sm);
+    strip_body<T, S, S / 4, S, VIA>(cr, d, n, ld, b, I0 + q * (S / 4), J0, last, reverse, nullptr, ap, bp_ld, via,
+                                    via_ld, sm);
   else
     strip_body<T, S, S, S / 4, VIA>(cr, d, n, ld, b, I0, J0 + q * (S / 4), last, reverse,
-                                    MODE == 1 ? bp : nullptr, bp_ld, via, via_ld, sm);
+                                    MODE == 1 ? bp : nullptr, nullptr, bp_ld, via, via_ld, sm);
 }
 
 }  // namespace apsp

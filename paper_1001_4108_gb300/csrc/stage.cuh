@@ -213,7 +213,7 @@ __device__ __forceinline__ void st_close(typename Arith<T>::C (&x)[4][4], typena
   }
 }
 
-// Two adjacent elements, read through L2 only; and written.
+// Two adjacent elements, read through L2 only.
 __device__ __forceinline__ void ld2cg(const float *p, float &x, float &y) {
   const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
   x = v.x;
@@ -229,12 +229,6 @@ __device__ __forceinline__ void ld2cg(const int16_t *p, int32_t &x, int32_t &y) 
   x = v.x;
   y = v.y;
 }
-__device__ __forceinline__ void st2(float *p, float x, float y) { *reinterpret_cast<float2 *>(p) = make_float2(x, y); }
-__device__ __forceinline__ void st2(int32_t *p, int32_t x, int32_t y) { *reinterpret_cast<int2 *>(p) = make_int2(x, y); }
-__device__ __forceinline__ void st2(int16_t *p, int16_t x, int16_t y) {
-  *reinterpret_cast<short2 *>(p) = make_short2(x, y);
-}
-
 // rest(b): phase 3 of stage b on the tiles outside rows and columns b, c: CTA t
 // of g.rest updates one 64 x 64 tile, 4 x 4 elements per thread; one more CTA
 // (t = g.rest) moves the closed diagonal tile of stage b to the matrix.  As, Bs:
