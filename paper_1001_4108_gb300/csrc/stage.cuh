@@ -284,6 +284,13 @@ __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typenam
           x[a][e + 1] = i < g.n && j + 1 < g.n ? Arith<T>::load(__ldcg(p + 1)) : Arith<T>::inf();
         }
       }
+    C x0[4][4];  // path bookkeeping: the values to be replaced
+    if (VIA) {
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x0[a][e] = x[a][e];
+    }
     const bool late = !mbar_wait_bounded(bar, 0);
     if (!late) st_product<C, 32, 2, 2, 128, 128, 64, 2>(x, As + 4 * ty, Bs + 4 * tx, g.one);
     if (__any_sync(0xffffffffu, late)) {  // give up: wait (bounded) for the copies in flight, store nothing
@@ -298,9 +305,8 @@ __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typenam
         for (int e = 0; e < 4; e += 2) {
           const int64_t i = i0 + st_idx(0, a), j = j0 + st_idx(0, e);
           if (VIA && g.via && i < g.n) {
-            const T *p = g.src + i * g.src_ld + j;
-            if (j < g.n) note_via(g.via, g.via_ld, i, j, x[a][e], Arith<T>::load(__ldcg(p)), b);
-            if (j + 1 < g.n) note_via(g.via, g.via_ld, i, j + 1, x[a][e + 1], Arith<T>::load(__ldcg(p + 1)), b);
+            if (j < g.n) note_via(g.via, g.via_ld, i, j, x[a][e], x0[a][e], b);
+            if (j + 1 < g.n) note_via(g.via, g.via_ld, i, j + 1, x[a][e + 1], x0[a][e + 1], b);
           }
           const T v0 = last ? Arith<T>::finish(x[a][e]) : (T)x[a][e];
           const T v1 = last ? Arith<T>::finish(x[a][e + 1]) : (T)x[a][e + 1];
@@ -550,7 +556,7 @@ __global__ void __launch_bounds__(kStThreads) __cluster_dims__(kStCluster, 1, 1)
 // (n = 1792 int32 590 us with the pad, 667 without).
 constexpr size_t kRestPad = 20 * 1024;
 template <typename T, bool VIA>
-__global__ void __launch_bounds__(kStThreads, 4) fw_rest(const StageArgs<T> g) {
+__global__ void __launch_bounds__(kStThreads, VIA ? 3 : 4) fw_rest(const StageArgs<T> g) {
   using C = typename Arith<T>::C;
   __shared__ __align__(128) C As[kStTile];
   __shared__ __align__(128) C Bs[kStTile];
