@@ -430,7 +430,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     const int R16 = (int)((n + S16 - 1) / S16);
     size_t ws16 = workspace_bytes_for(n, APSP_I16, S16);
     if (uses_stage_launches(S16, R16, true, a.flags, a.events != nullptr))
-      ws16 = std::max(ws16, stage_ws_bytes(R16));
+      ws16 = std::max(ws16, stage_ws_bytes(R16, true));
     size_t got = 0;
     char *buf = static_cast<char *>(
         library_workspace(dev, a.stream, copy_bytes + ws16, cap != cudaStreamCaptureStatusNone, &got));
@@ -462,7 +462,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   const size_t need = (a.flags & APSP_FLAG_NO_WORKSPACE) ? 0 : workspace_bytes_with(n, dtype, a.S, a.flags);
   const int R = (int)((n + a.S - 1) / a.S);
   const size_t stage_need =
-      uses_stage_launches(a.S, R, dtype == APSP_I16, a.flags, a.events != nullptr) ? stage_ws_bytes(R) : 0;
+      uses_stage_launches(a.S, R, dtype == APSP_I16, a.flags, a.events != nullptr) ? stage_ws_bytes(R, dtype == APSP_I16) : 0;
   // the int32 kernels that read both panels from copies, not the matrix
   constexpr int kNoPairs = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_WORKSPACE;
   const size_t pairs_need = stage_need || dtype != APSP_I32 || R < 2 || (a.flags & kNoPairs)

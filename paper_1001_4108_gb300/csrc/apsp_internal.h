@@ -85,17 +85,20 @@ inline bool uses_strips(int S, int R, bool f32, bool i16) {
 // requests (no forced kernel, plain schedule or tracing) and enough workspace,
 // up to the stage count at which its rest stops paying.  us per solve with the
 // lookahead schedule and with it: int32 n = 1300 489 and 339, 1664 565 and 503,
-// 2048 776 and 778, 3072 about 2000 and 2080; fp32 n = 1408 445 and 403, 1792
-// 612 and 629, 2048 952 and 822.  int16 is computed in 32 bits here, half the
-// packed kernels' rate: n = 1024 296 and 229, 1280 375 and 328, 1408 406 and 413.
-constexpr int kStageMaxRounds = 32, kStageMaxRoundsI16 = 21;
+// 2048 776 and 779, 3072 about 2000 and 2080; fp32 n = 1408 428 and 402, 1792
+// 611 and 612, 2048 850 and 823; int16 n = 512 154 and 110, 1024 296 and 229,
+// 1536 446 and 385, 2048 660 and 594, 2304 829 and 799, 2560 948 and 952.
+constexpr int kStageMaxRounds = 32, kStageMaxRoundsI16 = 36;
 inline bool uses_stage_launches(int S, int R, bool i16, int flags, bool traced) {
   constexpr int kOther = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_LOOKAHEAD | APSP_FLAG_NO_WORKSPACE;
   return S == 64 && R <= (i16 ? kStageMaxRoundsI16 : kStageMaxRounds) && !(flags & kOther) && !traced;
 }
 // Its workspace: two panel buffers (row and column, R tiles of 64 x 64 words
-// each) and two diagonal tiles.
-inline size_t stage_ws_bytes(int R) { return ((size_t)4 * R + 2) * 64 * 64 * sizeof(int32_t); }
+// each) and two diagonal tiles; int16 also two buffers of packed panels (R
+// tiles of 64 x 32 and 64 x 64 words).
+inline size_t stage_ws_bytes(int R, bool i16) {
+  return ((size_t)4 * R + 2 + (i16 ? (size_t)3 * R : 0)) * 64 * 64 * sizeof(int32_t);
+}
 
 // Workspace bytes of the packed int16x2 phase 3 (replicated column panel:
 // n_p rows x s words).

@@ -189,7 +189,7 @@ static int run_rounds(const RunArgs &a) {
   }
   // s = 64 without special requests: one launch per stage
   if constexpr (S == 64) {
-    if (uses_stage_launches(S, R, std::is_same<T, int16_t>::value, a.flags, a.events != nullptr) && a.ws && a.ws_bytes >= stage_ws_bytes(R) &&
+    if (uses_stage_launches(S, R, std::is_same<T, int16_t>::value, a.flags, a.events != nullptr) && a.ws && a.ws_bytes >= stage_ws_bytes(R, std::is_same<T, int16_t>::value) &&
         reinterpret_cast<uintptr_t>(a.ws) % 256 == 0)
       return run_stages<T, VIA>(a);
   }

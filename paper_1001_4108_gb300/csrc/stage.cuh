@@ -74,6 +74,14 @@ struct StageArgs {
   __device__ __forceinline__ C *row_panel(int stage) const { return ws + (size_t)(stage & 1) * 2 * R * kStTile; }
   __device__ __forceinline__ C *col_panel(int stage) const { return row_panel(stage) + (size_t)R * kStTile; }
   __device__ __forceinline__ C *diag(int stage) const { return ws + ((size_t)4 * R + (stage & 1)) * kStTile; }
+  // int16: the panels once more, as rest reads them: two columns per word, and
+  // rows with each entry in both halves of a word
+  __device__ __forceinline__ uint32_t *packed_row(int stage) const {
+    return reinterpret_cast<uint32_t *>(ws + ((size_t)4 * R + 2) * kStTile) + (size_t)(stage & 1) * 3 * R * (kStTile / 2);
+  }
+  __device__ __forceinline__ uint32_t *packed_col(int stage) const {
+    return packed_row(stage) + (size_t)R * (kStTile / 2);
+  }
 };
 
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
@@ -114,6 +122,12 @@ __device__ __forceinline__ int st_idx(int t, int a) { return 2 * t + 32 * (a >> 
 // kp0 .. kp0 + KP - 1.  A: rows of k pairs of AS words, the thread's row pairs
 // at a + 64 m (m < M); B: rows of BS words, its column pairs at b + BSTEP q
 // (q < Q).
+// C = uint32_t: two int16 columns per word (packed).
+template <> struct Vec4<uint32_t> { using V = uint4; };
+template <bool FMA>
+__device__ __forceinline__ uint32_t relax2(uint32_t acc, uint32_t a0, uint32_t a1, uint32_t b0, uint32_t b1, int) {
+  return __viaddmin_s16x2(a1, b1, __viaddmin_s16x2(a0, b0, acc));
+}
 template <typename C, int KP, int M, int Q, int AS, int BS, int BSTEP, int UN>
 __device__ __forceinline__ void st_product(C (&y)[2 * M][2 * Q], const C *a, const C *b, int one, int kp0 = 0) {
   using V = typename Vec4<C>::V;
@@ -229,6 +243,10 @@ __device__ __forceinline__ void ld2cg(const int16_t *p, int32_t &x, int32_t &y) 
   x = v.x;
   y = v.y;
 }
+template <bool VIA>
+__device__ __forceinline__ void stage_rest_packed(const StageArgs<int16_t> &g, int t, uint32_t *As, uint32_t *Bs,
+                                                  uint64_t *bar);
+
 // rest(b): phase 3 of stage b on the tiles outside rows and columns b, c: CTA t
 // of g.rest updates one 64 x 64 tile, 4 x 4 elements per thread; one more CTA
 // (t = g.rest) moves the closed diagonal tile of stage b to the matrix.  As, Bs:
@@ -254,6 +272,8 @@ __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typenam
       const int64_t i = c0 + e / S, j = c0 + e % S;
       if (i < g.n && j < g.n) g.d[i * g.ld + j] = last ? Arith<T>::finish(v[u]) : (T)v[u];
     }
+  } else if constexpr (std::is_same<T, int16_t>::value) {
+    stage_rest_packed<VIA>(g, t, reinterpret_cast<uint32_t *>(As), reinterpret_cast<uint32_t *>(Bs), bar);
   } else {
     // the tile rows (columns) of the launch are all but b and c, in order
     const int skip = c < R ? 2 : 1, nr = R - skip;
@@ -318,6 +338,78 @@ __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typenam
             if (j + 1 < g.n) p[1] = v1;
           }
         }
+    }
+  }
+}
+
+// rest(b) for int16, two columns per 32-bit word (DPX viaddmin.s16x2): weights
+// are >= 0 and sums fit in 16 bits.  Thread rows st_idx(ty, .), words 2 tx, 2 tx
+// + 1 (columns 4 tx .. 4 tx + 3).
+template <bool VIA>
+__device__ __forceinline__ void stage_rest_packed(const StageArgs<int16_t> &g, int t, uint32_t *As, uint32_t *Bs,
+                                                  uint64_t *bar) {
+  constexpr int S = kStS;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  const int b = g.b, R = g.R, c = b + 1;
+  const int skip = c < R ? 2 : 1, nr = R - skip;
+  const int tr = t / nr, tc = t - tr * nr;
+  const int I = tr < b ? tr : tr + skip, J = tc < b ? tc : tc + skip;
+  if (tid == 0) {
+    mbar_arrive_expect_tx(bar, (kStTile + kStTile / 2) * 4);
+    bulk_load(As, g.packed_col(b) + (size_t)I * kStTile, kStTile * 4, bar);
+    bulk_load(Bs, g.packed_row(b) + (size_t)J * (kStTile / 2), kStTile / 2 * 4, bar);
+  }
+  const int ty = 4 * (warp / 2) + lane / 8, tx = 8 * (warp % 2) + lane % 8;
+  const int64_t i0 = (int64_t)I * S + 2 * ty, j0 = (int64_t)J * S + 4 * tx;
+  const bool whole = (int64_t)(I + 1) * S <= g.n && (int64_t)(J + 1) * S <= g.n;
+  // whole tiles and rows that allow four columns per access
+  const bool quad = whole && reinterpret_cast<uintptr_t>(g.d) % 8 == 0 && g.ld % 4 == 0;
+  uint32_t x[4][2], x0[4][2];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int64_t i = i0 + st_idx(0, a);
+    const int16_t *p = g.d + i * g.ld + j0;
+    if (quad) {
+      const uint2 v = __ldcg(reinterpret_cast<const uint2 *>(p));
+      x[a][0] = v.x;
+      x[a][1] = v.y;
+    } else {
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const uint32_t lo = i < g.n && j0 + 2 * w < g.n ? (uint16_t)__ldcg(p + 2 * w) : 16383u;
+        const uint32_t hi = i < g.n && j0 + 2 * w + 1 < g.n ? (uint16_t)__ldcg(p + 2 * w + 1) : 16383u;
+        x[a][w] = lo | (hi << 16);
+      }
+    }
+  }
+  if (VIA) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int w = 0; w < 2; ++w) x0[a][w] = x[a][w];
+  }
+  const bool late = !mbar_wait_bounded(bar, 0);
+  if (!late) st_product<uint32_t, 32, 2, 1, 128, 64, 0, 4>(x, As + 4 * ty, Bs + 4 * tx, g.one);
+  if (__any_sync(0xffffffffu, late)) {  // give up: wait (bounded) for the copies in flight, store nothing
+    if (lane == 0) {
+      atomicCAS(g.err, 0, (int)kDevTimeoutTma);
+      mbar_wait_bounded(bar, 0);
+    }
+    return;
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int64_t i = i0 + st_idx(0, a);
+    int16_t *p = g.d + i * g.ld + j0;
+    if (quad) *reinterpret_cast<uint2 *>(p) = make_uint2(x[a][0], x[a][1]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int v = (int)(x[a][e / 2] >> (16 * (e % 2)) & 0xffffu);
+      if (i < g.n && j0 + e < g.n) {
+        if (VIA && g.via)
+          note_via(g.via, g.via_ld, i, j0 + e, v, (int)(x0[a][e / 2] >> (16 * (e % 2)) & 0xffffu), b);
+        if (!quad) p[e] = (int16_t)v;
+      }
     }
   }
 }
@@ -535,6 +627,21 @@ __global__ void __launch_bounds__(kStThreads) __cluster_dims__(kStCluster, 1, 1)
   for (int q = 0; q < Q; ++q)
     *reinterpret_cast<V *>(out + ry * 128 + 4 * sx + 32 * q) =
         V{z[0][2 * q], z[1][2 * q], z[0][2 * q + 1], z[1][2 * q + 1]};
+  if constexpr (std::is_same<T, int16_t>::value) {
+    const int xs = W * (u % kUnits);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      uint32_t v[4];  // (e, f) = (0, 0), (1, 0), (0, 1), (1, 1)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = (uint32_t)z[i & 1][2 * q + (i >> 1)] & 0xffffu;
+      if (cols)
+        *reinterpret_cast<uint4 *>(g.packed_col(c) + (size_t)J * kStTile + ry * 128 + 2 * xs + 4 * sx + 32 * q) =
+            make_uint4(v[0] * 0x10001u, v[1] * 0x10001u, v[2] * 0x10001u, v[3] * 0x10001u);
+      else
+        *reinterpret_cast<uint2 *>(g.packed_row(c) + (size_t)J * (kStTile / 2) + ry * 64 + xs + 2 * sx + 16 * q) =
+            make_uint2(v[0] | v[2] << 16, v[1] | v[3] << 16);
+    }
+  }
 #pragma unroll
   for (int e = 0; e < 2; ++e)
 #pragma unroll
@@ -578,21 +685,25 @@ __global__ void __launch_bounds__(kStThreads, VIA ? 3 : 4) fw_rest(const StageAr
 // has a handful of tiles (with more, the next stage's heads are placed two to
 // an SM).  Measured, us per solve: n = 768 int32 164 with W = 32, 173 with 16;
 // n = 512 fp32 104 with 16, 111 with 32; n = 1920 int32 676 with 32, 727 with
-// 64; n = 2048 int32 783 with 64, 822 with 32.  In one launch: n = 256 53 (57
+// 64; n = 2048 int32 779 with 64, 821 with 32, fp32 with unaligned rows 885 and
+// 1071, int16 676 and 594; n = 2304 int16 799 and 840.  In one launch: n = 256 53 (57
 // with two), n = 512 118 (104), n = 1024 323 (221).
 struct HeadCut {
   int W;        // strip width: 16, 32 or 64
   bool merged;  // rest(b) in the head's launch
 };
-inline HeadCut head_cut(int R) {
+inline HeadCut head_cut(int R, bool i16) {
   if (R <= 9) return {16, R <= 5};
-  if (R <= 30) return {32, false};
+  if (R <= (i16 ? 33 : 30)) return {32, false};
   return {64, false};
 }
 
 template <typename T, int W, bool VIA>
 static cudaError_t launch_head(const StageArgs<T> &g, int grid, cudaStream_t st) {
-  constexpr size_t smem = sizeof(HeadSmem<typename Arith<T>::C, W>) + 128;
+  // more than half of an SM's shared memory: the next stage's heads, launched
+  // while these run, must not end up two to an SM (n = 1792 int16 494 us, 586
+  // without, int32 574 and 587)
+  constexpr size_t smem = std::max<size_t>(sizeof(HeadSmem<typename Arith<T>::C, W>) + 128, 116 * 1024);
   static thread_local uint64_t done = 0;  // bit per device
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
@@ -627,7 +738,7 @@ static int run_stages(const RunArgs &a) {
   g.via_ld = a.via_ld;
   g.err = a.err;
   g.one = 1;
-  const HeadCut cut = head_cut(R);
+  const HeadCut cut = head_cut(R, std::is_same<T, int16_t>::value);
   g.half = std::max(1, S / cut.W * (R - 1));
   g.heads = (2 * g.half + kStCluster - 1) / kStCluster * kStCluster;
   for (int b = -1; b < (R == 1 ? 0 : R); ++b) {
