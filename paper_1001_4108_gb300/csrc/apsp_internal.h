@@ -83,7 +83,7 @@ inline bool uses_strips(int S, int R, bool f32, bool i16) {
 
 // One head and one rest per stage (stage.cuh), s = 64: calls without special
 // requests (no forced kernel, plain schedule or tracing) and enough workspace,
-// up to the stage count at which its rest stops paying.  us per solve with the
+// from two stages (one is a single fw_phase1) up to the count at which its rest stops paying.  us per solve with the
 // lookahead schedule and with it: int32 n = 1300 489 and 339, 1664 565 and 503,
 // 2048 776 and 779, 3072 about 2000 and 2080; fp32 n = 1408 428 and 402, 1792
 // 611 and 612, 2048 850 and 823; int16 n = 512 154 and 110, 1024 296 and 229,
@@ -91,7 +91,7 @@ inline bool uses_strips(int S, int R, bool f32, bool i16) {
 constexpr int kStageMaxRounds = 32, kStageMaxRoundsI16 = 36;
 inline bool uses_stage_launches(int S, int R, bool i16, int flags, bool traced) {
   constexpr int kOther = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_LOOKAHEAD | APSP_FLAG_NO_WORKSPACE;
-  return S == 64 && R <= (i16 ? kStageMaxRoundsI16 : kStageMaxRounds) && !(flags & kOther) && !traced;
+  return S == 64 && R >= 2 && R <= (i16 ? kStageMaxRoundsI16 : kStageMaxRounds) && !(flags & kOther) && !traced;
 }
 // Its workspace: two panel buffers (row and column, R tiles of 64 x 64 words
 // each) and two diagonal tiles; int16 also two buffers of packed panels (R

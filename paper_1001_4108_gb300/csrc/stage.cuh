@@ -568,8 +568,7 @@ __global__ void __launch_bounds__(kStThreads) __cluster_dims__(kStCluster, 1, 1)
       for (int e = 0; e < 4; ++e) {
         const int64_t i = c0 + st_idx(ty, a), j = c0 + st_idx(tx, e);
         if (VIA && g.via && i < g.n && j < g.n) note_via(g.via, g.via_ld, i, j, x[a][e], before[a][e], c);
-        if (R > 1) g.diag(c)[st_idx(ty, a) * S + st_idx(tx, e)] = x[a][e];
-        else if (i < g.n && j < g.n) g.d[i * g.ld + j] = Arith<T>::finish(x[a][e]);  // nothing else to do
+        g.diag(c)[st_idx(ty, a) * S + st_idx(tx, e)] = x[a][e];
       }
   }
   // the closed tile as an operand: D(i, k) for row panel strips, D(k, j) for column panel strips
@@ -722,7 +721,7 @@ static cudaError_t launch_head(const StageArgs<T> &g, int grid, cudaStream_t st)
   return launch(fw_head<T, W, VIA>, dim3(grid), kStThreads, smem, st, 0, g);
 }
 
-// All stages of one matrix with s = 64.  ws: stage_ws_bytes bytes, 16-byte
+// All stages of one matrix with s = 64 and two stages or more.  ws: stage_ws_bytes bytes, 16-byte
 // aligned.
 template <typename T, bool VIA>
 static int run_stages(const RunArgs &a) {
@@ -739,9 +738,9 @@ static int run_stages(const RunArgs &a) {
   g.err = a.err;
   g.one = 1;
   const HeadCut cut = head_cut(R, std::is_same<T, int16_t>::value);
-  g.half = std::max(1, S / cut.W * (R - 1));
+  g.half = S / cut.W * (R - 1);
   g.heads = (2 * g.half + kStCluster - 1) / kStCluster * kStCluster;
-  for (int b = -1; b < (R == 1 ? 0 : R); ++b) {
+  for (int b = -1; b < R; ++b) {
     g.b = b;
     g.src = b == 0 && a.first_src ? static_cast<const T *>(a.first_src) : g.d;
     g.src_ld = b == 0 && a.first_src ? a.first_src_ld : a.ld;

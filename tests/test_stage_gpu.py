@@ -2,7 +2,7 @@
 bit-identical to the plain schedule for any leading dimension and alignment,
 and to the oracle for the integers.
 
-The stage counts are the edges of its ranges: one stage; head and rest in one
+The stage counts are the edges of its ranges: one stage (fw_phase1); head and rest in one
 launch up to 5 stages; panel strips 16 wide up to 9 stages, 32 wide up to 30
 (int16: 33), then 64; the lookahead schedule beyond 32 (int16: 36) stages.  Whole and ragged last stages."""
 import numpy as np
