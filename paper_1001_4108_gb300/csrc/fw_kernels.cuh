@@ -723,15 +723,28 @@ __global__ void __launch_bounds__(P3Tma<S>::TPB, P3Tma<S>::MIN_BLOCKS)
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                      : "=f"(bq[m].x), "=f"(bq[m].y), "=f"(bq[m].z), "=f"(bq[m].w)
                      : "r"(smem_u32(B + p * (2 * S) + 4 * G * m)));
+      // s = 128: a row's sums, then its minima (n = 8192 29.01 ms; sum by sum
+      // 29.17).  s = 64: every second row's odd columns by two scalar adds
+      // (n = 4096 4.10 ms; packed adds only 4.23; at s = 128 29.58).
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
+      for (int r = 0; r < 8; ++r) {
+        float2 sum[8];
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-          const float2 s0 = add2f(ap[r], make_float2(bq[m].x, bq[m].y));
-          const float2 s1 = add2f(ap[r], make_float2(bq[m].z, bq[m].w));
-          acc[r][2 * m] = min3f(acc[r][2 * m], s0.x, s0.y);
-          acc[r][2 * m + 1] = min3f(acc[r][2 * m + 1], s1.x, s1.y);
+          const float2 b0 = make_float2(bq[m].x, bq[m].y), b1 = make_float2(bq[m].z, bq[m].w);
+          sum[2 * m] = add2f(ap[r], b0);
+          sum[2 * m + 1] = S == 64 && r % 2 == 0 ? make_float2(__fadd_rn(ap[r].x, b1.x), __fadd_rn(ap[r].y, b1.y))
+                                                 : add2f(ap[r], b1);
+          if (S == 64) {
+            acc[r][2 * m] = min3f(acc[r][2 * m], sum[2 * m].x, sum[2 * m].y);
+            acc[r][2 * m + 1] = min3f(acc[r][2 * m + 1], sum[2 * m + 1].x, sum[2 * m + 1].y);
+          }
         }
+        if (S != 64) {
+#pragma unroll
+          for (int c = 0; c < 8; ++c) acc[r][c] = min3f(acc[r][c], sum[c].x, sum[c].y);
+        }
+      }
     }
     // the last warp done with stage st refills it with slice s + STAGES (no
     // CTA barrier per slice, none at the end: 1.2 % faster than a barrier
