@@ -768,7 +768,7 @@ def roofline_block(dtype: str, n: int, m: dict, sms: int, peaks: dict, peak_kind
     p3_relax_mean = statistics.mean(p3_relax) if p3_relax else float("nan")
     hbm_bytes = 2.0 * m["es"] * p3_relax_mean / S  # C tile read + write per phase-3 launch
     return {"bound": "alu",
-            "kernel": {"f32": f"fw_phase3_f32x2<{S},...>", "i32": f"fw_tile_tma<int,{S},0>",
+            "kernel": {"f32": f"fw_phase3_f32x2<{S},...>", "i32": f"fw_phase3_pairs<{S},0>",
                        "i16": f"fw_tile_s16x2<{S},0>"}[dtype],
             "achieved": achieved, "peak": peak,
             "unit": "relaxations/s", "frac": achieved / peak,

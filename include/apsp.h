@@ -151,12 +151,16 @@ typedef struct apsp_config {
     int32_t phase3_tma;      /* 1 if the TMA-staged phase-3 kernel is used          */
     int32_t phase3_threads;  /* threads per phase-3 CTA                             */
     int64_t phase3_relax_per_round; /* relaxations phase 3 performs in a full round */
-    int32_t lookahead;       /* 1 if a call without flags uses the lookahead schedule
-                                (stages >= 3, TMA-staged kernels, library workspace) */
-    int32_t strips;          /* 1 if a call without flags on 16-byte aligned rows cuts
-                                each 64 x 64 tile of its phase-2 launches (and of the
-                                lookahead's cross launches) into four one-CTA strips:
-                                s = 64, fp32 up to 48 stages, int32 up to 32 */
+    int32_t lookahead;       /* 1 if the lookahead schedule is available (stages >= 3,
+                                TMA-staged kernels, library workspace).  With s = 64
+                                and 2 to 32 stages (int16: 36) a call without flags,
+                                tracing or a workspace of its own runs one head and
+                                one rest kernel per stage instead: same results */
+    int32_t strips;          /* 1 if the lookahead and plain schedules on 16-byte
+                                aligned rows cut each 64 x 64 tile of their phase-2
+                                launches (and of the lookahead's cross launches) into
+                                four one-CTA strips: s = 64, fp32 up to 48 stages,
+                                int32 up to 32 */
 } apsp_config;
 
 /* Status name, e.g. "APSP_EINVAL".  Never NULL. */
@@ -173,9 +177,13 @@ APSP_API int apsp_version(void);
  *   ld     leading dimension in elements, ld >= n.
  *   dtype  APSP_I32 / APSP_F32 / APSP_I16.
  *   stream cudaStream_t (cast to void*); NULL = legacy default stream.
- * Stream-ordered: returns after the work is enqueued.  The fast phase-3 path
- * needs dist 16-byte aligned and ld*sizeof(element) a multiple of 16; other
- * layouts run a generic kernel (same results, slower).
+ * Stream-ordered: returns after the work is enqueued.  The staged phase-3
+ * kernels need dist 16-byte aligned and ld*sizeof(element) a multiple of 16.
+ * Other layouts: up to 32 stages of s = 64 (int16: 36) the kernels take any
+ * layout; above, the matrix is solved on an aligned copy (n x n elements of
+ * device memory in stream order for the duration of the solve, from a pool of
+ * the library that keeps at most 64 MiB); without memory for it, or while the
+ * stream is being captured, a generic kernel runs (same results, slower).
  * Returns APSP_EINVAL on a bad argument, APSP_ECUDA if a launch fails.
  */
 APSP_API int apsp_fw(void *dist, int64_t n, int64_t ld, int dtype, void *stream);
@@ -248,7 +256,9 @@ APSP_API int apsp_path(const void *dist, const int16_t *via, int64_t n, int64_t 
  * From 3 stages on, two such buffers (the lookahead schedule writes the next
  * stage's copy while phase 3 reads the current one); a workspace holding one
  * buffer runs the plain schedule.  Without a workspace the same results come
- * from slower phase-3 kernels.
+ * from slower phase-3 kernels.  The workspaces the library owns can be larger
+ * (and int32 solves have one): both panels in copies of their own, at most
+ * 4 * s * ceil(n/s) * s * 4 bytes (7 in the place of 4 for int16 with s = 64).
  */
 APSP_API int64_t apsp_workspace_bytes(int64_t n, int dtype, int32_t kblock);
 
@@ -263,11 +273,12 @@ APSP_API int64_t apsp_workspace_bytes(int64_t n, int dtype, int32_t kblock);
  * The scratch the packed phase 3 needs (the interleaved row panel) lives in a
  * static device array of the library, 8 MiB, held by every GPU that loads the
  * library until the process exits.  Limit: n <= 16384; larger n returns
- * APSP_EUNSUPPORTED before any device work.  With dist 16-byte aligned, ld * 4
- * a multiple of 16 and n above one tile, the solve always runs the packed
- * kernels on the array (if they cannot run, the call returns
- * APSP_EUNSUPPORTED before any device work); other layouts run the unpacked
- * kernels, which need no scratch.  The first call on each device
+ * APSP_EUNSUPPORTED before any device work.  Up to 32 stages of s = 64 the
+ * solve runs one head and one rest kernel per stage on the array, in any
+ * layout.  Above, with dist 16-byte aligned and ld * 4 a multiple of 16, it
+ * always runs the packed kernels on the array (if they cannot run, the call
+ * returns APSP_EUNSUPPORTED before any device work); other layouts run the
+ * unpacked kernels, which need no scratch.  The first call on each device
  * looks up the array's device address (cudaGetSymbolAddress); make that first
  * call before any stream capture.  All calls share the one array and each
  * solve rewrites every part of it that it reads, so nothing needs clearing;

@@ -83,11 +83,12 @@ inline bool uses_strips(int S, int R, bool f32, bool i16) {
 
 // One head and one rest per stage (stage.cuh), s = 64: calls without special
 // requests (no forced kernel, plain schedule or tracing) and enough workspace,
-// from two stages (one is a single fw_phase1) up to the count at which its rest stops paying.  us per solve with the
-// lookahead schedule and with it: int32 n = 1300 489 and 339, 1664 565 and 503,
-// 2048 776 and 779, 3072 about 2000 and 2080; fp32 n = 1408 428 and 402, 1792
-// 611 and 612, 2048 850 and 823; int16 n = 512 154 and 110, 1024 296 and 229,
-// 1536 446 and 385, 2048 660 and 594, 2304 829 and 799, 2560 948 and 952.
+// from two stages on (one stage is a single fw_phase1) up to the count at which
+// its rest stops paying.  us per solve with the lookahead schedule and with it:
+// int32 n = 1280 395 and 349, 1536 473 and 446, 1792 585 and 588, 2048 778 and
+// 757; fp32 n = 1024 264 and 240, 1536 482 and 466, 1792 626 and 610, 2048 852
+// and 766; int16 n = 512 154 and 110, 1024 296 and 229, 1536 446 and 385, 2048
+// 660 and 594, 2304 829 and 799, 2560 948 and 952.
 constexpr int kStageMaxRounds = 32, kStageMaxRoundsI16 = 36;
 inline bool uses_stage_launches(int S, int R, bool i16, int flags, bool traced) {
   constexpr int kOther = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_LOOKAHEAD | APSP_FLAG_NO_WORKSPACE;

@@ -76,7 +76,8 @@ extern "C" int apsp_fw_f32_noalloc(void *dist, int64_t n, int64_t ld, void *stre
   a.ws = panel;
   a.ws_bytes = kPanelFloats * sizeof(float);
   // One panel buffer always fits (s * ceil(n/s) * s floats <= 128 * 16384),
-  // so the solve takes the plain schedule on the static array; whenever the
+  // so the solve takes the plain schedule on the static array (small ones the
+  // one-head-per-stage schedule, which fits as well); whenever the
   // layout allows the packed kernels they must use it (the run refuses
   // rather than fall back to the unpacked kernels without telling).
   if (apsp::interleaved_panel_bytes(n, a.S) > a.ws_bytes) return APSP_EUNSUPPORTED;

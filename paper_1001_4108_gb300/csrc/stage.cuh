@@ -568,7 +568,6 @@ __global__ void __launch_bounds__(kStThreads) __cluster_dims__(kStCluster, 1, 1)
       for (int e = 0; e < 4; ++e) {
         const int64_t i = c0 + st_idx(ty, a), j = c0 + st_idx(tx, e);
         if (VIA && g.via && i < g.n && j < g.n) note_via(g.via, g.via_ld, i, j, x[a][e], before[a][e], c);
-        g.diag(c)[st_idx(ty, a) * S + st_idx(tx, e)] = x[a][e];
       }
   }
   // the closed tile as an operand: D(i, k) for row panel strips, D(k, j) for column panel strips
@@ -584,6 +583,13 @@ __global__ void __launch_bounds__(kStThreads) __cluster_dims__(kStCluster, 1, 1)
             V{x[2 * m][2 * q], x[2 * m][2 * q + 1], x[2 * m + 1][2 * q], x[2 * m + 1][2 * q + 1]};
     }
 
+  if (lead) {  // here and in pairs: 4 % of an int32 n = 1024 solve against word stores before the operand's
+    C *dg = g.diag(c);
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int e = 0; e < 4; e += 2) st2(dg + st_idx(ty, a) * S + st_idx(tx, e), x[a][e], x[a][e + 1]);
+  }
   if (!has) return;
   if (helps) {  // the strip after stage b
     if (VIA && g.via && upd) {
