@@ -428,12 +428,14 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     const int S16 = choose_kblock(n, APSP_I16, opt ? opt->kblock : 0);
     const size_t copy_bytes = ((size_t)n * ld16 * 2 + 255) / 256 * 256;
     const int R16 = (int)((n + S16 - 1) / S16);
-    size_t ws16 = workspace_bytes_for(n, APSP_I16, S16);
-    if (uses_stage_launches(S16, R16, true, a.flags, a.events != nullptr))
-      ws16 = std::max(ws16, stage_ws_bytes(R16, true));
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    const size_t least16 = workspace_bytes_for(n, APSP_I16, S16);
+    const bool staged = uses_stage_launches(S16, R16, APSP_I16, false, a.flags, a.events != nullptr);
+    const size_t ws16 = staged ? std::max(least16, stage_ws_bytes(R16, true)) : least16;
     size_t got = 0;
-    char *buf = static_cast<char *>(
-        library_workspace(dev, a.stream, copy_bytes + ws16, cap != cudaStreamCaptureStatusNone, &got));
+    void *mem = library_workspace(dev, a.stream, copy_bytes + ws16, capturing, &got);
+    if (!mem && least16 < ws16) mem = library_workspace(dev, a.stream, copy_bytes + least16, capturing, &got);
+    char *buf = static_cast<char *>(mem);
     if (buf) {  // else (first use inside a capture): the int32 path, same result
       if (narrow_to_i16(static_cast<const int32_t *>(dist), n, ld, reinterpret_cast<int16_t *>(buf), ld16,
                         a.stream) != APSP_OK)
@@ -443,8 +445,8 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       b.ld = ld16;
       b.S = S16;
       b.tma_ok = true;  // 256-byte aligned buffer, 16-byte rows
-      b.ws = ws16 ? buf + copy_bytes : nullptr;
       b.ws_bytes = ws16 ? got - copy_bytes : 0;
+      b.ws = b.ws_bytes ? buf + copy_bytes : nullptr;
       if (!(b.flags & APSP_FLAG_NO_LOOKAHEAD)) {
         std::lock_guard<std::mutex> lk(g_mu);
         side_resources_locked(dev, b.stream, cap != cudaStreamCaptureStatusNone, &b);
@@ -462,7 +464,9 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   const size_t need = (a.flags & APSP_FLAG_NO_WORKSPACE) ? 0 : workspace_bytes_with(n, dtype, a.S, a.flags);
   const int R = (int)((n + a.S - 1) / a.S);
   const size_t stage_need =
-      uses_stage_launches(a.S, R, dtype == APSP_I16, a.flags, a.events != nullptr) ? stage_ws_bytes(R, dtype == APSP_I16) : 0;
+      uses_stage_launches(a.S, R, dtype, via != nullptr, a.flags, a.events != nullptr)
+          ? stage_ws_bytes(R, dtype == APSP_I16)
+          : 0;
   // the int32 kernels that read both panels from copies, not the matrix
   constexpr int kNoPairs = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_WORKSPACE;
   const size_t pairs_need = stage_need || dtype != APSP_I32 || R < 2 || (a.flags & kNoPairs)
@@ -482,8 +486,9 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       a.ws = opt->workspace;
       a.ws_bytes = (size_t)opt->workspace_bytes;
     } else {
-      a.ws = library_workspace(dev, a.stream, std::max(need, more), cap != cudaStreamCaptureStatusNone,
-                               &a.ws_bytes);
+      const bool capturing = cap != cudaStreamCaptureStatusNone;
+      a.ws = library_workspace(dev, a.stream, std::max(need, more), capturing, &a.ws_bytes);
+      if (!a.ws && need && need < more) a.ws = library_workspace(dev, a.stream, need, capturing, &a.ws_bytes);
       if (!a.ws) a.ws_bytes = 0;  // the kernels fall back to the form that needs none
     }
   }
@@ -496,10 +501,16 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     return APSP_ECUDA;
   const bool direct = (a.flags & APSP_FLAG_NO_GRAPH) || a.events || cap != cudaStreamCaptureStatusNone;
   // Rows that are not 16-byte aligned: the staged kernels work on an aligned
-  // copy (two passes over the matrix, against kernels two to four times slower;
-  // the one-launch-per-stage schedule takes any layout by itself).
+  // copy (two passes over the matrix, against kernels two to four times slower).
+  // The one-launch-per-stage schedule takes any layout by itself, at word loads
+  // and stores of the matrix in each stage: below kStageCopyRounds stages these
+  // cost less than the copies, us in place and with them: fp32 n = 1025 270 and
+  // 285, 1281 406 and 408, 1537 561 and 527, 2047 872 and 800, 3073 2585 and
+  // 2289; int32 1025 264 and 277, 1537 522 and 511, 2047 831 and 788; int16
+  // 1025 255 and 266, 1537 487 and 442, 2047 775 and 641.
+  constexpr int kStageCopyRounds = 22;
   constexpr int kInPlace = APSP_FLAG_GENERIC | APSP_FLAG_NO_WORKSPACE;
-  const bool any_layout = stage_need && a.ws_bytes >= stage_need;
+  const bool any_layout = stage_need && a.ws_bytes >= stage_need && R < kStageCopyRounds;
   void *copy = nullptr;
   const int64_t cld = (n * (int64_t)es + 15) / 16 * 16 / (int64_t)es;
   if (!a.tma_ok && !any_layout && R > 1 && !(a.flags & kInPlace) && cap == cudaStreamCaptureStatusNone)

@@ -86,13 +86,22 @@ inline bool uses_strips(int S, int R, bool f32, bool i16) {
 // from two stages on (one stage is a single fw_phase1) up to the count at which
 // its rest stops paying.  us per solve with the lookahead schedule and with it:
 // int32 n = 1280 395 and 349, 1536 473 and 446, 1792 585 and 588, 2048 778 and
-// 757; fp32 n = 1024 264 and 240, 1536 482 and 466, 1792 626 and 610, 2048 852
-// and 766; int16 n = 512 154 and 110, 1024 296 and 229, 1536 446 and 385, 2048
-// 660 and 594, 2304 829 and 799, 2560 948 and 952.
-constexpr int kStageMaxRounds = 32, kStageMaxRoundsI16 = 36;
-inline bool uses_stage_launches(int S, int R, bool i16, int flags, bool traced) {
+// 757, 2304 1078 and 940, 2496 1227 and 1185, 2560 1310 and 1311; fp32 n = 1024
+// 264 and 240, 1536 482 and 466, 2048 852 and 766, 2304 1192 and 998, 2816 1843
+// and 1629, 3328 2606 and 2551, 3584 3046 and 3127; int16 n = 512 154 and 110,
+// 1024 296 and 229, 1536 446 and 385, 2048 660 and 594, 2304 829 and 799, 2560
+// 948 and 952.  With the stage record (via) the other schedule's bulk kernel
+// is further behind: fp32 n = 2304 1864 and 1276, 3072 3605 and 2562, 4096 6865
+// and 5681; int32 2304 1673 and 1208, 3072 2906 and 2468, 3584 4323 and 3774,
+// 4032 6383 and 5377; int16 2560 1397 and 1153, 3072 1980 and 1775, 4032 3827 and
+// 3632; fp32 5056 (79 stages) 10477 and 9482.
+inline int stage_max_rounds(bool f32, bool i16, bool via) {
+  return via ? (f32 ? 80 : 64) : (f32 ? 52 : i16 ? 36 : 39);
+}
+inline bool uses_stage_launches(int S, int R, int dtype, bool via, int flags, bool traced) {
   constexpr int kOther = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_LOOKAHEAD | APSP_FLAG_NO_WORKSPACE;
-  return S == 64 && R >= 2 && R <= (i16 ? kStageMaxRoundsI16 : kStageMaxRounds) && !(flags & kOther) && !traced;
+  return S == 64 && R >= 2 && R <= stage_max_rounds(dtype == APSP_F32, dtype == APSP_I16, via) &&
+         !(flags & kOther) && !traced;
 }
 // Its workspace: two panel buffers (row and column, R tiles of 64 x 64 words
 // each) and two diagonal tiles; int16 also two buffers of packed panels (R

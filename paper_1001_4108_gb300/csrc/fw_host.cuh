@@ -189,8 +189,10 @@ static int run_rounds(const RunArgs &a) {
   }
   // s = 64 without special requests: one launch per stage
   if constexpr (S == 64) {
-    if (uses_stage_launches(S, R, std::is_same<T, int16_t>::value, a.flags, a.events != nullptr) && a.ws && a.ws_bytes >= stage_ws_bytes(R, std::is_same<T, int16_t>::value) &&
-        reinterpret_cast<uintptr_t>(a.ws) % 256 == 0)
+    constexpr bool kI16 = std::is_same<T, int16_t>::value;
+    constexpr int kType = kI16 ? APSP_I16 : std::is_same<T, float>::value ? APSP_F32 : APSP_I32;
+    if (uses_stage_launches(S, R, kType, a.via != nullptr, a.flags, a.events != nullptr) && a.ws &&
+        a.ws_bytes >= stage_ws_bytes(R, kI16) && reinterpret_cast<uintptr_t>(a.ws) % 256 == 0)
       return run_stages<T, VIA>(a);
   }
   const cudaStream_t st = a.stream;

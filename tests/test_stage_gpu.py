@@ -4,7 +4,9 @@ and to the oracle for the integers.
 
 The stage counts are the edges of its ranges: one stage (fw_phase1); head and rest in one
 launch up to 5 stages; panel strips 16 wide up to 9 stages, 32 wide up to 30
-(int16: 33), then 64; the lookahead schedule beyond 32 (int16: 36) stages.  Whole and ragged last stages."""
+(int16: 33), then 64; the lookahead schedule beyond 52 (fp32), 39 (int32) and 36 (int16) stages, with
+the stage record beyond 80, 64 and 64.  Whole and ragged last stages.  Rows that are not 16-byte aligned
+go through an aligned copy from 22 stages on."""
 import numpy as np
 import pytest
 
@@ -96,3 +98,50 @@ def test_stage_schedule_capture_and_replay(n):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(d, ref)
+
+
+@pytest.mark.parametrize("dt,n,paths", [
+    ("f32", 3265, False), ("f32", 3328, False), ("f32", 3329, False), ("i32", 2433, False), ("i32", 2496, False),
+    ("i32", 2497, False), ("i16", 2304, False), ("f32", 5120, True), ("f32", 5121, True), ("i32", 4096, True),
+    ("i32", 4097, True), ("i16", 4033, True), ("i16", 4097, True)])
+def test_stage_schedule_last_rounds(dt, n, paths):
+    w = graph(dt, n, n + 3)
+    a, b = on_device(w, (n + 7) // 8 * 8), on_device(w, (n + 7) // 8 * 8)
+    plain = binding.FLAG_NO_LOOKAHEAD | binding.FLAG_NO_GRAPH
+    if paths:
+        va, vb = (torch.empty((n, n), dtype=torch.int16, device="cuda") for _ in range(2))
+        binding.apsp_fw_paths(a, va, n, kblock=64)
+        binding.apsp_fw_paths(b, vb, n, kblock=64, flags=plain)
+        assert torch.equal(va, vb)
+    else:
+        binding.apsp_fw(a, n)
+        binding.apsp_fw(b, n, flags=plain)
+    assert torch.equal(a, b)
+    assert binding.device_error() == 0
+
+
+@pytest.mark.parametrize("dt", ["f32", "i32", "i16"])
+@pytest.mark.parametrize("n", [1344, 1345, 2047])
+def test_stage_schedule_unaligned_copy(dt, n):
+    # in place below 22 stages, an aligned copy from there on, in place again under capture
+    w = graph(dt, n, n + 4)
+    ref = on_device(w, (n + 7) // 8 * 8)
+    vr, v = (torch.empty((n, n), dtype=torch.int16, device="cuda") for _ in range(2))
+    binding.apsp_fw_paths(ref, vr, n)
+    s = torch.cuda.Stream()
+    d = on_device(w, n + 9, 1)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        binding.apsp_fw_paths(d, v, n, stream=s)
+    torch.cuda.synchronize()
+    assert torch.equal(d[:, :n], ref[:, :n]) and torch.equal(v, vr)
+    assert bool((d[:, n:] == -7).all())
+    g = torch.cuda.CUDAGraph()
+    d[:, :n] = torch.from_numpy(w).cuda()
+    v.fill_(7)
+    with torch.cuda.graph(g, stream=s):
+        binding.apsp_fw_paths(d, v, n, stream=s)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(d[:, :n], ref[:, :n]) and torch.equal(v, vr)
+    assert bool((d[:, n:] == -7).all())
