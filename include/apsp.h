@@ -153,7 +153,8 @@ typedef struct apsp_config {
     int64_t phase3_relax_per_round; /* relaxations phase 3 performs in a full round */
     int32_t lookahead;       /* 1 if the lookahead schedule is available (stages >= 3,
                                 TMA-staged kernels, library workspace).  With s = 64
-                                and 2 to 32 stages (int16: 36) a call without flags,
+                                and 2 to 52 (fp32), 39 (int32) or 36 (int16) stages,
+                                apsp_fw_paths up to 80, 64 and 64, a call without flags,
                                 tracing or a workspace of its own runs one head and
                                 one rest kernel per stage instead: same results */
     int32_t strips;          /* 1 if the lookahead and plain schedules on 16-byte
@@ -179,11 +180,13 @@ APSP_API int apsp_version(void);
  *   stream cudaStream_t (cast to void*); NULL = legacy default stream.
  * Stream-ordered: returns after the work is enqueued.  The staged phase-3
  * kernels need dist 16-byte aligned and ld*sizeof(element) a multiple of 16.
- * Other layouts: up to 32 stages of s = 64 (int16: 36) the kernels take any
- * layout; above, the matrix is solved on an aligned copy (n x n elements of
+ * Other layouts: below 22 stages of s = 64 the kernels take any layout; from
+ * there on the matrix is solved on an aligned copy (n x n elements of
  * device memory in stream order for the duration of the solve, from a pool of
  * the library that keeps at most 64 MiB); without memory for it, or while the
- * stream is being captured, a generic kernel runs (same results, slower).
+ * stream is being captured, it is solved in place (same results, slower: the
+ * kernels for any layout up to the stage counts of apsp_config.lookahead, a
+ * generic kernel above).
  * Returns APSP_EINVAL on a bad argument, APSP_ECUDA if a launch fails.
  */
 APSP_API int apsp_fw(void *dist, int64_t n, int64_t ld, int dtype, void *stream);
@@ -273,7 +276,7 @@ APSP_API int64_t apsp_workspace_bytes(int64_t n, int dtype, int32_t kblock);
  * The scratch the packed phase 3 needs (the interleaved row panel) lives in a
  * static device array of the library, 8 MiB, held by every GPU that loads the
  * library until the process exits.  Limit: n <= 16384; larger n returns
- * APSP_EUNSUPPORTED before any device work.  Up to 32 stages of s = 64 the
+ * APSP_EUNSUPPORTED before any device work.  Up to 52 stages of s = 64 the
  * solve runs one head and one rest kernel per stage on the array, in any
  * layout.  Above, with dist 16-byte aligned and ld * 4 a multiple of 16, it
  * always runs the packed kernels on the array (if they cannot run, the call
