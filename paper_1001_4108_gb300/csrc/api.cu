@@ -8,6 +8,7 @@
 
 #include "../../include/apsp.h"
 #include "apsp_internal.h"
+#include "graph_key.h"
 
 // Device error word: bounded waits that give up record a code here.
 static __device__ int g_apsp_err;
@@ -137,25 +138,8 @@ void side_resources_locked(int dev, cudaStream_t stream, bool capturing, RunArgs
 // ---------------------------------------------------------------- graphs
 // A solve is 3 launches per stage (4 with the lookahead's split phase 3).
 // Replaying them as one CUDA graph removes the per-launch host cost, which
-// dominates for small n.  A graph is captured the
-// second time the same (matrix, n, ld, dtype, s, flags) is solved, so one-off
-// calls do not pay the instantiation.
-struct GraphKey {
-  void *d;
-  int64_t n, ld;
-  int dtype, S, flags, dev;
-  cudaStream_t stream;
-  void *ws;
-  void *via;
-  int64_t via_ld;
-  const void *first_src;
-  void *last_dst;
-  bool operator==(const GraphKey &o) const {
-    return d == o.d && n == o.n && ld == o.ld && dtype == o.dtype && S == o.S && flags == o.flags &&
-           dev == o.dev && stream == o.stream && ws == o.ws && via == o.via && via_ld == o.via_ld &&
-           first_src == o.first_src && last_dst == o.last_dst;
-  }
-};
+// dominates for small n.  A graph is captured the second time the same solve
+// (GraphKey) is asked for, so one-off calls do not pay the instantiation.
 struct GraphEntry {
   GraphKey key;
   cudaGraphExec_t exec;
@@ -167,8 +151,7 @@ std::vector<GraphKey> g_seen;
 cudaStream_t g_capture_stream[kMaxDev];
 
 int launch_with_graph(const RunArgs &a, int dtype, int dev) {
-  const GraphKey key{a.d, a.n, a.ld, dtype, a.S, a.flags, dev, a.stream, a.ws, a.via, a.via_ld, a.first_src,
-                     a.last_dst};
+  const GraphKey key = graph_key(a, dtype, dev);
   std::lock_guard<std::mutex> lk(g_mu);
   for (auto &g : g_graphs)
     if (g.key == key) return cudaGraphLaunch(g.exec, a.stream) == cudaSuccess ? APSP_OK : APSP_ECUDA;
