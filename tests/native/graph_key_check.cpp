@@ -38,6 +38,8 @@ static void differs(const char *what, F &&change) {
 
 int main() {
   differs("the workspace's size", [](RunArgs &b) { b.ws_bytes = 0; });
+  differs("the host matrix's leading dimension (in)", [](RunArgs &b) { b.first_src_ld += 64; });
+  differs("the host matrix's leading dimension (out)", [](RunArgs &b) { b.last_dst_ld += 64; });
   std::printf(fails ? "%d failed checks\n" : "ok\n", fails);
   return fails ? 1 : 0;
 }
