@@ -9,6 +9,7 @@
 #include "../../include/apsp.h"
 #include "apsp_internal.h"
 #include "graph_key.h"
+#include "workspace.h"
 
 // Device error word: bounded waits that give up record a code here.
 static __device__ int g_apsp_err;
@@ -188,21 +189,10 @@ int launch_with_graph(const RunArgs &a, int dtype, int dev) {
   return cudaGraphLaunch(exec, a.stream) == cudaSuccess ? APSP_OK : APSP_ECUDA;
 }
 
-// Library-owned workspaces, one per (device, stream): work on one stream is
-// ordered, so a stream's solves can share one buffer.  Allocated outside of
-// stream capture only; grown on demand.
-struct WsEntry {
-  int dev;
-  cudaStream_t stream;
-  void *p;
-  size_t bytes;
-};
-constexpr size_t kMaxWs = 16;
-std::vector<WsEntry> g_ws;
-
 // Graphs captured with a workspace bake its address in: drop them before the
-// buffer is freed.  Caller holds g_mu.
+// buffer is freed.
 void forget_graphs_using(void *ws) {
+  std::lock_guard<std::mutex> lk(g_mu);
   for (size_t i = 0; i < g_graphs.size();) {
     if (g_graphs[i].key.ws == ws) {
       cudaGraphExecDestroy(g_graphs[i].exec);
@@ -215,38 +205,7 @@ void forget_graphs_using(void *ws) {
                g_seen.end());
 }
 
-void *library_workspace(int dev, cudaStream_t stream, size_t bytes, bool capturing, size_t *got) {
-  std::lock_guard<std::mutex> lk(g_mu);
-  for (auto &e : g_ws)
-    if (e.dev == dev && e.stream == stream) {
-      if (e.bytes >= bytes) {
-        *got = e.bytes;
-        return e.p;
-      }
-      if (capturing) return nullptr;
-      cudaDeviceSynchronize();
-      forget_graphs_using(e.p);
-      cudaFree(e.p);
-      e.p = nullptr;
-      e.bytes = 0;
-      if (cudaMalloc(&e.p, bytes) != cudaSuccess) return nullptr;
-      e.bytes = bytes;
-      *got = bytes;
-      return e.p;
-    }
-  if (capturing) return nullptr;
-  if (g_ws.size() >= kMaxWs) {
-    cudaDeviceSynchronize();
-    forget_graphs_using(g_ws.front().p);
-    cudaFree(g_ws.front().p);
-    g_ws.erase(g_ws.begin());
-  }
-  void *p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
-  g_ws.push_back({dev, stream, p, bytes});
-  *got = bytes;
-  return p;
-}
+Workspaces g_workspaces(forget_graphs_using);
 
 // One panel copy (fp32 interleaved row panel, int16 replicated column panel).
 size_t panel_bytes_for(int64_t n, int dtype, int S) {
@@ -299,11 +258,7 @@ void *copy_buffer(int dev, size_t bytes, cudaStream_t stream) {
     pool = g_copy_pool[dev];
   }
   void *p = nullptr;
-  if (cudaMallocFromPoolAsync(&p, bytes, pool, stream) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  return p;
+  return got_memory(cudaMallocFromPoolAsync(&p, bytes, pool, stream)) ? p : nullptr;
 }
 
 // Device buffer of apsp_fw_host, one per device, grown on demand.
@@ -416,8 +371,8 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     const bool staged = uses_stage_launches(S16, R16, APSP_I16, false, a.flags, a.events != nullptr);
     const size_t ws16 = staged ? std::max(least16, stage_ws_bytes(R16, true)) : least16;
     size_t got = 0;
-    void *mem = library_workspace(dev, a.stream, copy_bytes + ws16, capturing, &got);
-    if (!mem && least16 < ws16) mem = library_workspace(dev, a.stream, copy_bytes + least16, capturing, &got);
+    void *mem = g_workspaces.get(dev, a.stream, copy_bytes + ws16, capturing, &got);
+    if (!mem && least16 < ws16) mem = g_workspaces.get(dev, a.stream, copy_bytes + least16, capturing, &got);
     char *buf = static_cast<char *>(mem);
     if (buf) {  // else (first use inside a capture): the int32 path, same result
       if (narrow_to_i16(static_cast<const int32_t *>(dist), n, ld, reinterpret_cast<int16_t *>(buf), ld16,
@@ -470,8 +425,8 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       a.ws_bytes = (size_t)opt->workspace_bytes;
     } else {
       const bool capturing = cap != cudaStreamCaptureStatusNone;
-      a.ws = library_workspace(dev, a.stream, std::max(need, more), capturing, &a.ws_bytes);
-      if (!a.ws && need && need < more) a.ws = library_workspace(dev, a.stream, need, capturing, &a.ws_bytes);
+      a.ws = g_workspaces.get(dev, a.stream, std::max(need, more), capturing, &a.ws_bytes);
+      if (!a.ws && need && need < more) a.ws = g_workspaces.get(dev, a.stream, need, capturing, &a.ws_bytes);
       if (!a.ws) a.ws_bytes = 0;  // the kernels fall back to the form that needs none
     }
   }
@@ -582,7 +537,7 @@ extern "C" int apsp_fw_host(void *host_dist, int64_t n, int64_t ld, int dtype, v
       hs.buf = nullptr;
       hs.bytes = 0;
     }
-    if (cudaMalloc(&hs.buf, bytes) != cudaSuccess) return APSP_ENOMEM;
+    if (!got_memory(cudaMalloc(&hs.buf, bytes))) return APSP_ENOMEM;
     hs.bytes = bytes;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);

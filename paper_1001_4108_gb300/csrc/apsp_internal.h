@@ -10,6 +10,14 @@
 
 namespace apsp {
 
+// Whether an allocation succeeded.  A failed one leaves no error behind: the
+// launch checks that follow, in this call or a later one, read the runtime's
+// last error.
+inline bool got_memory(cudaError_t e) {
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess;
+}
+
 struct RunArgs {
   void *d;            // device matrix
   int64_t n, ld;      // vertices, leading dimension (elements)

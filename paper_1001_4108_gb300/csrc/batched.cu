@@ -262,7 +262,7 @@ int run_batched_small(const BatchDesc *host_descs, int count, int dtype, cudaStr
       e->groups.back().count = i + 1 - e->groups.back().first;
     }
     const size_t bytes = (size_t)count * sizeof(BatchDesc) + 16 * kMaxGroups;
-    if (cudaMalloc(&e->dev_buf, bytes) != cudaSuccess) {
+    if (!got_memory(cudaMalloc(&e->dev_buf, bytes))) {
       delete e;
       return APSP_ENOMEM;
     }
@@ -309,7 +309,7 @@ int run_batched_direct(const BatchDesc *host_descs, int count, int dtype, cudaSt
     *cap = 0;
     size_t c = 4096;
     while (c < need) c <<= 1;
-    if (cudaMallocAsync(dev_buf, c, st) != cudaSuccess) return APSP_ENOMEM;
+    if (!got_memory(cudaMallocAsync(dev_buf, c, st))) return APSP_ENOMEM;
     *cap = c;
   }
   // pageable source: the runtime stages it before returning

@@ -231,7 +231,7 @@ void launch_admitted(Server *s, std::vector<Request *> &adm) {
     const size_t si = s->next_stream;
     s->next_stream = 1 + (s->next_stream % (s->streams.size() - 1));
     cudaStream_t st = s->streams[si];
-    int rc = cudaMallocAsync(&r->dev, r->bytes, st) == cudaSuccess ? APSP_OK : APSP_ENOMEM;
+    int rc = got_memory(cudaMallocAsync(&r->dev, r->bytes, st)) ? APSP_OK : APSP_ENOMEM;
     if (rc == APSP_OK && cudaMemcpyAsync(r->dev, r->host, r->bytes, cudaMemcpyHostToDevice, st) != cudaSuccess)
       rc = APSP_ECUDA;
     if (rc == APSP_OK) {
@@ -258,7 +258,7 @@ void launch_admitted(Server *s, std::vector<Request *> &adm) {
     std::stable_sort(grp.begin(), grp.end(), [](Request *a, Request *b) { return a->n > b->n; });
     int rc = APSP_OK;
     for (Request *r : grp) {
-      if (rc == APSP_OK && cudaMallocAsync(&r->dev, r->bytes, st) != cudaSuccess) rc = APSP_ENOMEM;
+      if (rc == APSP_OK && !got_memory(cudaMallocAsync(&r->dev, r->bytes, st))) rc = APSP_ENOMEM;
       if (rc == APSP_OK && cudaMemcpyAsync(r->dev, r->host, r->bytes, cudaMemcpyHostToDevice, st) != cudaSuccess)
         rc = APSP_ECUDA;
     }
@@ -400,7 +400,7 @@ extern "C" int apsp_server_create(apsp_server **out, const apsp_server_config *c
     cudaStream_t st = nullptr;
     void *ws = nullptr;
     if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) rc = APSP_ECUDA;
-    if (rc == APSP_OK && s->ws_bytes && cudaMalloc(&ws, (size_t)s->ws_bytes) != cudaSuccess) rc = APSP_ENOMEM;
+    if (rc == APSP_OK && s->ws_bytes && !got_memory(cudaMalloc(&ws, (size_t)s->ws_bytes))) rc = APSP_ENOMEM;
     s->streams.push_back(st);
     s->workspaces.push_back(ws);
   }
@@ -446,7 +446,7 @@ extern "C" int apsp_submit(apsp_server *h, const void *host_dist, int64_t n, int
     std::lock_guard<std::mutex> lk(s->mu);
     pinned_take(s, std::max<size_t>(r->bytes, 1), &r->host, &r->host_cap);
   }
-  if (!r->host && cudaMallocHost(&r->host, r->host_cap) != cudaSuccess) {
+  if (!r->host && !got_memory(cudaMallocHost(&r->host, r->host_cap))) {
     delete r;
     return APSP_ENOMEM;
   }

@@ -120,8 +120,8 @@ extern "C" int apsp_autotune(int dtype, void *stream, char *report, int64_t repo
       total += (size_t)(n * n);
     }
     char *mats = nullptr, *meta = nullptr;
-    if (cudaMalloc(&mats, total * es) != cudaSuccess) return APSP_ENOMEM;
-    if (cudaMalloc(&meta, (size_t)count * sizeof(BatchDesc) + 16) != cudaSuccess) {
+    if (!got_memory(cudaMalloc(&mats, total * es))) return APSP_ENOMEM;
+    if (!got_memory(cudaMalloc(&meta, (size_t)count * sizeof(BatchDesc) + 16))) {
       cudaFree(mats);
       return APSP_ENOMEM;
     }
@@ -172,7 +172,7 @@ extern "C" int apsp_autotune(int dtype, void *stream, char *report, int64_t repo
       total += (size_t)(n * n);
     }
     char *mats = nullptr;
-    if (cudaMalloc(&mats, total * es) != cudaSuccess) return APSP_ENOMEM;
+    if (!got_memory(cudaMalloc(&mats, total * es))) return APSP_ENOMEM;
     size_t off = 0;
     for (auto &dsc : descs) {
       dsc.d = mats + off * es;
@@ -228,7 +228,7 @@ extern "C" int apsp_autotune(int dtype, void *stream, char *report, int64_t repo
   for (int i = 0; i < 5; ++i) {
     const int64_t n = sizes[i];
     char *m = nullptr;
-    if (cudaMalloc(&m, (size_t)n * n * es) != cudaSuccess) return APSP_ENOMEM;
+    if (!got_memory(cudaMalloc(&m, (size_t)n * n * es))) return APSP_ENOMEM;
     float ms[2] = {0, 0};
     int rc = APSP_OK;
     for (int j = 0; j < 2 && rc == APSP_OK; ++j) {
