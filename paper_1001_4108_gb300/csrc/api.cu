@@ -191,18 +191,20 @@ int launch_with_graph(const RunArgs &a, int dtype, int dev) {
 
 // Graphs captured with a workspace bake its address in: drop them before the
 // buffer is freed.
-void forget_graphs_using(void *ws) {
+void forget_graphs_using(void *p, size_t bytes) {
   std::lock_guard<std::mutex> lk(g_mu);
+  auto uses = [&](const GraphKey &k) {
+    return k.ws >= p && k.ws < static_cast<char *>(p) + bytes;
+  };
   for (size_t i = 0; i < g_graphs.size();) {
-    if (g_graphs[i].key.ws == ws) {
+    if (uses(g_graphs[i].key)) {
       cudaGraphExecDestroy(g_graphs[i].exec);
       g_graphs.erase(g_graphs.begin() + i);
     } else {
       ++i;
     }
   }
-  g_seen.erase(std::remove_if(g_seen.begin(), g_seen.end(), [&](const GraphKey &k) { return k.ws == ws; }),
-               g_seen.end());
+  g_seen.erase(std::remove_if(g_seen.begin(), g_seen.end(), uses), g_seen.end());
 }
 
 Workspaces g_workspaces(forget_graphs_using);
@@ -232,34 +234,8 @@ size_t workspace_bytes_with(int64_t n, int dtype, int S, int flags) {
   return bytes;
 }
 
-// Pool of the aligned copies of unaligned matrices (solve()), one per device;
-// memory above the threshold goes back to the device when nothing uses it.
-constexpr uint64_t kCopyPoolKeep = 64ull << 20;
-cudaMemPool_t g_copy_pool[kMaxDev];
-
-// A buffer in stream order; nullptr if there is none to be had.
-void *copy_buffer(int dev, size_t bytes, cudaStream_t stream) {
-  cudaMemPool_t pool;
-  {
-    std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_copy_pool[dev]) {
-      cudaMemPoolProps props{};
-      props.allocType = cudaMemAllocationTypePinned;
-      props.location.type = cudaMemLocationTypeDevice;
-      props.location.id = dev;
-      uint64_t keep = kCopyPoolKeep;
-      if (cudaMemPoolCreate(&g_copy_pool[dev], &props) != cudaSuccess ||
-          cudaMemPoolSetAttribute(g_copy_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-        cudaGetLastError();
-        g_copy_pool[dev] = nullptr;
-        return nullptr;
-      }
-    }
-    pool = g_copy_pool[dev];
-  }
-  void *p = nullptr;
-  return got_memory(cudaMallocFromPoolAsync(&p, bytes, pool, stream)) ? p : nullptr;
-}
+// Aligned copies of unaligned matrices (solve()).
+StreamPool g_copies(64ull << 20);
 
 // Device buffer of apsp_fw_host, one per device, grown on demand.
 struct HostStage {
@@ -370,11 +346,10 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     const size_t least16 = workspace_bytes_for(n, APSP_I16, S16);
     const bool staged = uses_stage_launches(S16, R16, APSP_I16, false, a.flags, a.events != nullptr);
     const size_t ws16 = staged ? std::max(least16, stage_ws_bytes(R16, true)) : least16;
-    size_t got = 0;
-    void *mem = g_workspaces.get(dev, a.stream, copy_bytes + ws16, capturing, &got);
-    if (!mem && least16 < ws16) mem = g_workspaces.get(dev, a.stream, copy_bytes + least16, capturing, &got);
-    char *buf = static_cast<char *>(mem);
-    if (buf) {  // else (first use inside a capture): the int32 path, same result
+    Workspaces::Lease mem =
+        g_workspaces.take(dev, a.stream, copy_bytes + ws16, copy_bytes + least16, capturing);
+    if (mem) {  // else (first use inside a capture): the int32 path, same result
+      char *buf = static_cast<char *>(mem.p);
       if (narrow_to_i16(static_cast<const int32_t *>(dist), n, ld, reinterpret_cast<int16_t *>(buf), ld16,
                         a.stream) != APSP_OK)
         return APSP_ECUDA;
@@ -383,7 +358,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       b.ld = ld16;
       b.S = S16;
       b.tma_ok = true;  // 256-byte aligned buffer, 16-byte rows
-      b.ws_bytes = ws16 ? got - copy_bytes : 0;
+      b.ws_bytes = ws16 ? mem.bytes - copy_bytes : 0;
       b.ws = b.ws_bytes ? buf + copy_bytes : nullptr;
       if (!(b.flags & APSP_FLAG_NO_LOOKAHEAD)) {
         std::lock_guard<std::mutex> lk(g_mu);
@@ -395,6 +370,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       if (widen_from_i16(reinterpret_cast<const int16_t *>(buf), ld16, n, static_cast<int32_t *>(dist), ld,
                          a.stream) != APSP_OK)
         return APSP_ECUDA;
+      mem.release();
       if (a.flags & APSP_FLAG_NEGCYCLE) return check_negcycle(dist, n, ld, dtype, a.stream, neg);
       return APSP_OK;
     }
@@ -411,6 +387,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
                                 ? 0
                                 : (R >= kLookaheadMinRounds ? 4 : 2) * interleaved_panel_bytes(n, a.S);
   const size_t more = std::max(stage_need, pairs_need);
+  Workspaces::Lease lease;  // until everything is enqueued
   if (need || more) {
     if (opt && opt->workspace && !need) {
       // not asked for: taken if it is enough for the kernels that can use one
@@ -424,10 +401,9 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       a.ws = opt->workspace;
       a.ws_bytes = (size_t)opt->workspace_bytes;
     } else {
-      const bool capturing = cap != cudaStreamCaptureStatusNone;
-      a.ws = g_workspaces.get(dev, a.stream, std::max(need, more), capturing, &a.ws_bytes);
-      if (!a.ws && need && need < more) a.ws = g_workspaces.get(dev, a.stream, need, capturing, &a.ws_bytes);
-      if (!a.ws) a.ws_bytes = 0;  // the kernels fall back to the form that needs none
+      lease = g_workspaces.take(dev, a.stream, std::max(need, more), need, cap != cudaStreamCaptureStatusNone);
+      a.ws = lease.p;  // none: the kernels fall back to the form that needs none
+      a.ws_bytes = lease.bytes;
     }
   }
   if (!(a.flags & APSP_FLAG_NO_LOOKAHEAD)) {
@@ -452,7 +428,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   void *copy = nullptr;
   const int64_t cld = (n * (int64_t)es + 15) / 16 * 16 / (int64_t)es;
   if (!a.tma_ok && !any_layout && R > 1 && !(a.flags & kInPlace) && cap == cudaStreamCaptureStatusNone)
-    copy = copy_buffer(dev, (size_t)n * cld * es, a.stream);
+    copy = g_copies.alloc(dev, (size_t)n * cld * es, a.stream);
   if (copy) {
     if (copy_matrix(dist, ld, copy, cld, n, (int)es, a.stream) != APSP_OK) st = APSP_ECUDA;
     a.d = copy;
@@ -465,6 +441,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     if (cudaFreeAsync(copy, a.stream) != cudaSuccess && st == APSP_OK) st = APSP_ECUDA;
   }
   if (st != APSP_OK) return st;
+  lease.release();
   if (a.flags & APSP_FLAG_NEGCYCLE) return check_negcycle(dist, n, ld, dtype, a.stream, neg);
   return APSP_OK;
 }

@@ -1,10 +1,13 @@
 // Host check of the library's workspaces (csrc/workspace.h) on a stand-in for
 // the CUDA runtime: this file defines the runtime functions that the header
 // calls.  Exit status 0 when every check holds; each failure is printed.
+#include <atomic>
 #include <cstdio>
 #include <map>
 #include <mutex>
 #include <set>
+#include <thread>
+#include <vector>
 
 #include "../../paper_1001_4108_gb300/csrc/workspace.h"
 
@@ -16,8 +19,9 @@ std::mutex mu;
 std::map<void *, size_t> live;
 size_t limit = 1u << 30, used = 0;
 cudaError_t last_error = cudaSuccess;
-int syncs = 0;
-std::set<void *> forgotten;
+std::atomic<int> syncs{0};
+int freed_leased = 0;
+std::set<void *> forgotten, leased;
 
 cudaError_t take(void **p, size_t bytes) {
   std::lock_guard<std::mutex> lk(mu);
@@ -31,12 +35,16 @@ cudaError_t give(void *p) {
   std::lock_guard<std::mutex> lk(mu);
   auto it = live.find(p);
   if (it == live.end()) return last_error = cudaErrorInvalidValue;
+  if (leased.count(p)) ++freed_leased;
   used -= it->second;
   live.erase(it);
   ::operator delete(p);
   return cudaSuccess;
 }
-void forget(void *p) { forgotten.insert(p); }
+void forget(void *p, size_t) {
+  std::lock_guard<std::mutex> lk(mu);
+  forgotten.insert(p);
+}
 cudaStream_t stream(int i) { return reinterpret_cast<cudaStream_t>((uintptr_t)0x1000 + 16 * i); }
 
 int fails = 0;
@@ -54,6 +62,13 @@ cudaError_t cudaDeviceSynchronize() {
   ++syncs;
   return cudaSuccess;
 }
+cudaError_t cudaMemPoolCreate(cudaMemPool_t *pool, const cudaMemPoolProps *) {
+  *pool = reinterpret_cast<cudaMemPool_t>((uintptr_t)0x10);
+  return cudaSuccess;
+}
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
+cudaError_t cudaMallocFromPoolAsync(void **p, size_t bytes, cudaMemPool_t, cudaStream_t) { return take(p, bytes); }
+cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return give(p); }
 cudaError_t cudaGetLastError() {
   const cudaError_t e = last_error;
   last_error = cudaSuccess;
@@ -63,35 +78,69 @@ cudaError_t cudaGetLastError() {
 
 static void reuse_and_growth() {
   Workspaces w(forget);
-  size_t got = 0;
-  void *a = w.get(0, stream(1), 1000, false, &got);
-  check(a && got == 1000, "a first buffer");
-  check(w.get(0, stream(1), 500, false, &got) == a && got == 1000, "a smaller request reuses it");
-  check(w.get(0, stream(2), 500, false, &got) != a, "another stream has its own");
-  void *b = w.get(0, stream(1), 2000, false, &got);
-  check(b && got == 2000, "a larger request");
+  void *a = nullptr;
+  {
+    Workspaces::Lease l = w.take(0, stream(1), 1000, 0, false);
+    check(l && l.bytes == 1000, "a first buffer");
+    a = l.p;
+  }
+  check(w.take(0, stream(1), 500, 0, false).p == a, "a smaller request reuses it");
+  check(w.take(0, stream(2), 500, 0, false).p != a, "another stream has its own");
+  check(w.take(1, stream(1), 500, 0, false).p != a, "so has another device");
+  check(w.take(0, stream(1), 2000, 0, false).bytes == 2000, "a larger request");
   check(forgotten.count(a) == 1, "graphs that use the old buffer are dropped");
 }
 
-// No memory: nullptr, the caller may ask for less, and no error stays behind.
+// No memory: less or none, and no error stays behind.
 static void out_of_memory() {
   Workspaces w(forget);
-  size_t got = 0;
   const size_t before = limit;
-  check(w.get(0, stream(1), 100, false, &got) != nullptr, "a small buffer");
+  check((bool)w.take(0, stream(1), 100, 0, false), "a small buffer");
   limit = used + 400;
-  check(w.get(0, stream(1), 1000, false, &got) == nullptr, "no memory for a larger one");
+  check(w.take(0, stream(1), 1000, 300, false).bytes == 300, "no memory for a larger one: the smaller size");
   check(last_error == cudaSuccess, "a failed allocation leaves an error for the launch checks");
-  check(w.get(0, stream(1), 300, false, &got) != nullptr && got == 300, "a smaller one is to be had");
+  check(!w.take(0, stream(1), 2000, 1000, false), "no memory");
   limit = used;
-  check(w.get(0, stream(2), 1, false, &got) == nullptr && last_error == cudaSuccess, "no memory on a new stream");
+  check(!w.take(0, stream(2), 1, 0, false) && last_error == cudaSuccess, "no memory on a new stream");
   limit = before;
-  check(w.get(0, stream(2), 1, false, &got) != nullptr && got == 1, "a later call finds memory");
+  check(w.take(0, stream(2), 1, 0, false).bytes == 1, "a later call finds memory");
+}
+
+// Threads: while one holds a lease, its buffer is neither freed nor handed to
+// another, whatever the others ask for; more streams than entries.
+static void threads() {
+  Workspaces w(forget);
+  std::atomic<int> freed{0}, shared{0}, none{0};
+  auto client = [&](int t, int s) {
+    for (int i = 0; i < 200; ++i) {
+      Workspaces::Lease l = w.take(0, stream(s), 100 + 37 * ((i + t) % 5) * (1 + i / 20), 0, false);
+      if (!l) {
+        ++none;
+        continue;
+      }
+      {
+        std::lock_guard<std::mutex> lk(mu);
+        if (!live.count(l.p)) ++freed;
+        if (!leased.insert(l.p).second) ++shared;
+      }
+      std::this_thread::yield();
+      std::lock_guard<std::mutex> lk(mu);
+      if (!live.count(l.p)) ++freed;
+      leased.erase(l.p);
+    }
+  };
+  std::vector<std::thread> th;
+  for (int t = 0; t < 40; ++t) th.emplace_back(client, t, t % 20);  // 20 streams, two threads each
+  for (auto &x : th) x.join();
+  check(freed == 0 && freed_leased == 0, "a buffer was freed while a thread held it");
+  check(shared == 0, "two threads held one buffer");
+  check(none == 0, "a stream found no memory");
 }
 
 int main() {
   reuse_and_growth();
   out_of_memory();
+  threads();
   std::printf(fails ? "%d failed checks\n" : "ok\n", fails);
   return fails ? 1 : 0;
 }
