@@ -108,15 +108,12 @@ class Workspaces {
     if (const std::shared_ptr<Entry> e = entry(dev, stream, !capturing)) {
       l.lk_ = std::unique_lock<std::mutex>(e->mu);
       if (e->bytes < bytes && !capturing) {
+        // in stream order: all work that uses the buffer is on this stream
         if (e->p) {
-          cudaDeviceSynchronize();
           forget_(e->p, e->bytes);
-          cudaFree(e->p);
+          cudaFreeAsync(e->p, stream);
         }
-        e->p = nullptr;
-        e->bytes = 0;
-        for (const size_t want : {bytes, least})
-          if (!e->p && want && got_memory(cudaMalloc(&e->p, want))) e->bytes = want;
+        e->bytes = alloc(dev, stream, bytes, least, &e->p);
       }
       if (e->bytes >= bytes || (least && e->bytes >= least)) {
         l.p = e->p;
@@ -126,9 +123,7 @@ class Workspaces {
         l.lk_.unlock();
       }
     } else if (!capturing) {
-      // more streams than entries: a buffer for this call, in stream order
-      for (const size_t want : {bytes, least})
-        if (!l.p && want && (l.p = spare_.alloc(dev, want, stream))) l.bytes = want;
+      l.bytes = alloc(dev, stream, bytes, least, &l.p);  // more streams than entries: a buffer for this call
     }
     return l;
   }
@@ -147,10 +142,17 @@ class Workspaces {
     entries_.push_back(e);
     return e;
   }
+  // `bytes` or else `least` bytes in *p; the size, 0 (*p = nullptr) without memory
+  size_t alloc(int dev, cudaStream_t stream, size_t bytes, size_t least, void **p) {
+    for (const size_t want : {bytes, least})
+      if (want && (*p = pool_.alloc(dev, want, stream))) return want;
+    *p = nullptr;
+    return 0;
+  }
   void (*forget_)(void *, size_t);
   std::mutex mu_;
   std::vector<std::shared_ptr<Entry>> entries_;
-  StreamPool spare_{64ull << 20};
+  StreamPool pool_{64ull << 20};
 };
 
 }  // namespace apsp

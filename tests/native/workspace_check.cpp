@@ -57,7 +57,10 @@ void check(bool ok, const char *what) {
 
 extern "C" {
 cudaError_t cudaMalloc(void **p, size_t bytes) { return take(p, bytes); }
-cudaError_t cudaFree(void *p) { return give(p); }
+cudaError_t cudaFree(void *p) {
+  ++syncs;  // waits for all work of the device
+  return give(p);
+}
 cudaError_t cudaDeviceSynchronize() {
   ++syncs;
   return cudaSuccess;
@@ -89,6 +92,8 @@ static void reuse_and_growth() {
   check(w.take(1, stream(1), 500, 0, false).p != a, "so has another device");
   check(w.take(0, stream(1), 2000, 0, false).bytes == 2000, "a larger request");
   check(forgotten.count(a) == 1, "graphs that use the old buffer are dropped");
+  for (int i = 3; i < 40; ++i) w.take(0, stream(i), 1000 * i, 0, false);
+  check(syncs == 0, "growing buffers and many streams synchronize the device");
 }
 
 // No memory: less or none, and no error stays behind.
