@@ -96,8 +96,9 @@ typedef enum apsp_status {
                                      solved by the packed int16x2 kernels (about twice the
                                      rate) and copied back, with absent = 2^29 in and out.
                                      Same results as the int32 path.  Uses library memory
-                                     (n^2 x 2 bytes + int16 panels, per device and stream);
-                                     APSP_EINVAL with a caller workspace or apsp_fw_paths. */
+                                     (n^2 x 2 bytes + int16 panels, per device and stream
+                                     or captured graph); APSP_EINVAL with a caller workspace
+                                     or apsp_fw_paths. */
 #define APSP_FLAG_ONE_LAUNCH 0x100 /* small matrices (s = 64, 2 to 32 stages): every
                                      stage in one cooperative launch, the tiles spread
                                      over the CTAs and ordered by per-tile flags in the
@@ -139,7 +140,11 @@ typedef struct apsp_options {
        only between the enqueue and the completion of this call's work on its
        stream; smaller: APSP_EINVAL.
        NULL = the library uses a buffer of its own, one per (device, stream),
-       allocated on first use (not while the stream is being captured). */
+       allocated on first use.  A solve in a stream capture gets a buffer that
+       belongs to the captured graph (shared by the solves captured on one
+       stream in it) and is given back when the graph and what was made from
+       it are destroyed: captured graphs share none of it with each other or
+       with later calls, and can be launched on any stream. */
     void *workspace;
     int64_t workspace_bytes;
 } apsp_options;

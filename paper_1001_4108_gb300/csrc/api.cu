@@ -33,8 +33,6 @@ EncodeTiledFn encode_tiled_fn() {
 
 namespace {
 
-constexpr int kMaxDev = 64;
-
 std::mutex g_mu;
 int *g_err_ptr[kMaxDev];
 int *g_neg_ptr[kMaxDev];
@@ -342,13 +340,12 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     const int S16 = choose_kblock(n, APSP_I16, opt ? opt->kblock : 0);
     const size_t copy_bytes = ((size_t)n * ld16 * 2 + 255) / 256 * 256;
     const int R16 = (int)((n + S16 - 1) / S16);
-    const bool capturing = cap != cudaStreamCaptureStatusNone;
     const size_t least16 = workspace_bytes_for(n, APSP_I16, S16);
     const bool staged = uses_stage_launches(S16, R16, APSP_I16, false, a.flags, a.events != nullptr);
     const size_t ws16 = staged ? std::max(least16, stage_ws_bytes(R16, true)) : least16;
     Workspaces::Lease mem =
-        g_workspaces.take(dev, a.stream, copy_bytes + ws16, copy_bytes + least16, capturing);
-    if (mem) {  // else (first use inside a capture): the int32 path, same result
+        g_workspaces.take(dev, a.stream, copy_bytes + ws16, copy_bytes + least16);
+    if (mem) {  // else: the int32 path, same result
       char *buf = static_cast<char *>(mem.p);
       if (narrow_to_i16(static_cast<const int32_t *>(dist), n, ld, reinterpret_cast<int16_t *>(buf), ld16,
                         a.stream) != APSP_OK)
@@ -401,7 +398,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       a.ws = opt->workspace;
       a.ws_bytes = (size_t)opt->workspace_bytes;
     } else {
-      lease = g_workspaces.take(dev, a.stream, std::max(need, more), need, cap != cudaStreamCaptureStatusNone);
+      lease = g_workspaces.take(dev, a.stream, std::max(need, more), need);
       a.ws = lease.p;  // none: the kernels fall back to the form that needs none
       a.ws_bytes = lease.bytes;
     }

@@ -1,8 +1,14 @@
-// Scratch memory that the library owns: one buffer per (device, stream), since
-// work on one stream is ordered and a stream's solves can share one.  Host code
-// only.
+// Scratch memory that the library owns.  Host code only.
+//
+// Work on one stream is ordered, so a stream's solves share one buffer per
+// (device, stream).  A solve in a caller's stream capture can not: its graph
+// may be launched on any stream, at any time, long after the stream's buffer
+// was outgrown.  Each capture has buffers of its own, which its graph (and
+// whatever is instantiated, cloned or updated from it) holds as a CUDA user
+// object; once the last of them is gone the memory goes back to the pool.
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 #include <memory>
 #include <mutex>
@@ -13,19 +19,33 @@
 
 namespace apsp {
 
+constexpr int kMaxDev = 64;
+
+// While it lives, this thread may allocate and wait although some thread's
+// stream capture forbids it: nothing here belongs to a capture.
+class OutsideCapture {
+ public:
+  OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+  ~OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+  OutsideCapture(const OutsideCapture &) = delete;
+
+ private:
+  cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+};
+
 // Device memory in stream order, from one pool per device.  Memory above
 // `keep` bytes goes back to the device when nothing uses it.
 class StreamPool {
  public:
   explicit StreamPool(uint64_t keep) : keep_(keep) {}
   void *alloc(int dev, size_t bytes, cudaStream_t stream) {
+    const OutsideCapture guard;
     const cudaMemPool_t pool = of(dev);
     void *p = nullptr;
     return pool && got_memory(cudaMallocFromPoolAsync(&p, bytes, pool, stream)) ? p : nullptr;
   }
 
  private:
-  static constexpr int kMaxDev = 64;
   cudaMemPool_t of(int dev) {
     std::lock_guard<std::mutex> lk(mu_);
     if (!pool_[dev]) {
@@ -53,6 +73,8 @@ class Workspaces {
     std::mutex mu;  // held from take() until the work that uses the buffer is enqueued
     void *p = nullptr;
     size_t bytes = 0;
+    unsigned long long capture = 0;  // the capture whose graph holds the buffer
+    std::atomic<bool> unused{false}; // that graph and its offspring are gone
   };
 
  public:
@@ -99,13 +121,23 @@ class Workspaces {
   explicit Workspaces(void (*forget)(void *, size_t)) : forget_(forget) {}
 
   // At least `bytes` bytes for work on `stream`, else at least `least` (if not
-  // 0), else an empty lease: there is no memory, or the stream is being
-  // captured and has no buffer of that size yet.  The caller then runs kernels
+  // 0), else an empty lease: there is no memory.  The caller then runs kernels
   // that need less or none.
-  Lease take(int dev, cudaStream_t stream, size_t bytes, size_t least, bool capturing) {
+  Lease take(int dev, cudaStream_t stream, size_t bytes, size_t least) {
     Lease l;
     l.stream_ = stream;
-    if (const std::shared_ptr<Entry> e = entry(dev, stream, !capturing)) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long capture = 0;
+    cudaGraph_t graph = nullptr;
+    if (cudaStreamGetCaptureInfo(stream, &status, &capture, &graph, nullptr, nullptr, nullptr) != cudaSuccess ||
+        status == cudaStreamCaptureStatusInvalidated) {
+      cudaGetLastError();
+      return l;
+    }
+    give_back(dev);
+    const bool capturing = status == cudaStreamCaptureStatusActive;
+    if (const std::shared_ptr<Entry> e =
+            capturing ? captured(dev, stream, capture, graph, bytes, least) : entry(dev, stream)) {
       l.lk_ = std::unique_lock<std::mutex>(e->mu);
       if (e->bytes < bytes && !capturing) {
         // in stream order: all work that uses the buffer is on this stream
@@ -115,7 +147,7 @@ class Workspaces {
         }
         e->bytes = alloc(dev, stream, bytes, least, &e->p);
       }
-      if (e->bytes >= bytes || (least && e->bytes >= least)) {
+      if (e->p) {
         l.p = e->p;
         l.bytes = e->bytes;
         l.entry_ = e;
@@ -131,16 +163,78 @@ class Workspaces {
  private:
   static constexpr size_t kMaxEntries = 16;
   // Entries are never evicted: another stream's work may be using the buffer.
-  std::shared_ptr<Entry> entry(int dev, cudaStream_t stream, bool create) {
+  std::shared_ptr<Entry> entry(int dev, cudaStream_t stream) {
     std::lock_guard<std::mutex> lk(mu_);
     for (auto &e : entries_)
       if (e->dev == dev && e->stream == stream) return e;
-    if (!create || entries_.size() >= kMaxEntries) return nullptr;
+    if (entries_.size() >= kMaxEntries) return nullptr;
     auto e = std::make_shared<Entry>();
     e->dev = dev;
     e->stream = stream;
     entries_.push_back(e);
     return e;
+  }
+  // The buffer of the solves that are captured on `stream` into `graph`, one
+  // after the other; nullptr without memory.
+  std::shared_ptr<Entry> captured(int dev, cudaStream_t stream, unsigned long long capture, cudaGraph_t graph,
+                                  size_t bytes, size_t least) {
+    std::lock_guard<std::mutex> lk(mu_);
+    for (auto &e : captured_)
+      if (e->capture == capture && e->stream == stream && e->dev == dev && e->bytes >= bytes) return e;
+    const OutsideCapture guard;
+    const cudaStream_t home = home_stream(dev);
+    if (!home) return nullptr;
+    auto e = std::make_shared<Entry>();
+    e->dev = dev;
+    e->stream = stream;
+    e->capture = capture;
+    for (const size_t want : {bytes, least})
+      if (!e->p && want && (e->p = capture_pool_.alloc(dev, want, home))) e->bytes = want;
+    if (!e->p) return nullptr;
+    auto *held = new std::shared_ptr<Entry>(e);
+    cudaUserObject_t object = nullptr;
+    const bool made =
+        cudaUserObjectCreate(&object, held, &graph_gone, 1, cudaUserObjectNoDestructorSync) == cudaSuccess;
+    if (!made) delete held;
+    // the memory is there before any launch of the graph
+    if (!made || cudaStreamSynchronize(home) != cudaSuccess ||
+        cudaGraphRetainUserObject(graph, object, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+      cudaGetLastError();
+      if (made) cudaUserObjectRelease(object, 1);
+      cudaFreeAsync(e->p, home);
+      return nullptr;
+    }
+    captured_.push_back(e);
+    return e;
+  }
+  // Runs on a thread of the CUDA runtime when nothing refers to a capture's
+  // graph any more: no CUDA calls in here.
+  static void CUDART_CB graph_gone(void *held) {
+    auto *e = static_cast<std::shared_ptr<Entry> *>(held);
+    (*e)->unused = true;
+    ++unused_;
+    delete e;
+  }
+  // Returns the buffers of captures that are gone to their pool.
+  void give_back(int dev) {
+    if (unused_ == 0) return;
+    const OutsideCapture guard;
+    std::lock_guard<std::mutex> lk(mu_);
+    for (size_t i = 0; i < captured_.size();) {
+      if (captured_[i]->unused && captured_[i]->dev == dev) {
+        cudaFreeAsync(captured_[i]->p, home_[dev]);
+        captured_.erase(captured_.begin() + i);
+        --unused_;
+      } else {
+        ++i;
+      }
+    }
+  }
+  // The stream of the captures' allocations: nothing else runs on it.
+  cudaStream_t home_stream(int dev) {
+    if (!home_[dev] && !got_memory(cudaStreamCreateWithFlags(&home_[dev], cudaStreamNonBlocking)))
+      home_[dev] = nullptr;
+    return home_[dev];
   }
   // `bytes` or else `least` bytes in *p; the size, 0 (*p = nullptr) without memory
   size_t alloc(int dev, cudaStream_t stream, size_t bytes, size_t least, void **p) {
@@ -153,6 +247,10 @@ class Workspaces {
   std::mutex mu_;
   std::vector<std::shared_ptr<Entry>> entries_;
   StreamPool pool_{64ull << 20};
+  std::vector<std::shared_ptr<Entry>> captured_;
+  static inline std::atomic<int> unused_{0};  // entries of captured_ whose graph is gone
+  StreamPool capture_pool_{64ull << 20};
+  cudaStream_t home_[kMaxDev] = {};
 };
 
 }  // namespace apsp

@@ -7,6 +7,7 @@
 #include <mutex>
 #include <set>
 #include <thread>
+#include <utility>
 #include <vector>
 
 #include "../../paper_1001_4108_gb300/csrc/workspace.h"
@@ -22,6 +23,9 @@ cudaError_t last_error = cudaSuccess;
 std::atomic<int> syncs{0};
 int freed_leased = 0;
 std::set<void *> forgotten, leased;
+std::map<cudaStream_t, unsigned long long> capturing;            // stream -> capture, also its graph
+std::map<unsigned long long, std::vector<cudaUserObject_t>> held;  // graph -> its objects
+bool refuse_objects = false;
 
 cudaError_t take(void **p, size_t bytes) {
   std::lock_guard<std::mutex> lk(mu);
@@ -72,6 +76,46 @@ cudaError_t cudaMemPoolCreate(cudaMemPool_t *pool, const cudaMemPoolProps *) {
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
 cudaError_t cudaMallocFromPoolAsync(void **p, size_t bytes, cudaMemPool_t, cudaStream_t) { return take(p, bytes); }
 cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return give(p); }
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *mode) {
+  thread_local cudaStreamCaptureMode current = cudaStreamCaptureModeGlobal;
+  std::swap(*mode, current);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
+  *s = stream(99);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+  if (s != stream(99)) ++syncs;
+  return cudaSuccess;
+}
+cudaError_t cudaStreamGetCaptureInfo(cudaStream_t s, cudaStreamCaptureStatus *status, unsigned long long *id,
+                                     cudaGraph_t *graph, const cudaGraphNode_t **, const cudaGraphEdgeData **,
+                                     size_t *) {
+  std::lock_guard<std::mutex> lk(mu);
+  auto it = capturing.find(s);
+  *status = it == capturing.end() ? cudaStreamCaptureStatusNone : cudaStreamCaptureStatusActive;
+  if (it != capturing.end()) {
+    *id = it->second;
+    *graph = reinterpret_cast<cudaGraph_t>((uintptr_t)it->second);
+  }
+  return cudaSuccess;
+}
+cudaError_t cudaUserObjectCreate(cudaUserObject_t *o, void *p, cudaHostFn_t destroy, unsigned, unsigned) {
+  *o = reinterpret_cast<cudaUserObject_t>(new std::pair<cudaHostFn_t, void *>(destroy, p));
+  return cudaSuccess;
+}
+cudaError_t cudaUserObjectRelease(cudaUserObject_t o, unsigned) {
+  auto *x = reinterpret_cast<std::pair<cudaHostFn_t, void *> *>(o);
+  x->first(x->second);
+  delete x;
+  return cudaSuccess;
+}
+cudaError_t cudaGraphRetainUserObject(cudaGraph_t g, cudaUserObject_t o, unsigned, unsigned) {
+  if (refuse_objects) return last_error = cudaErrorInvalidValue;
+  held[(unsigned long long)reinterpret_cast<uintptr_t>(g)].push_back(o);
+  return cudaSuccess;
+}
 cudaError_t cudaGetLastError() {
   const cudaError_t e = last_error;
   last_error = cudaSuccess;
@@ -83,16 +127,16 @@ static void reuse_and_growth() {
   Workspaces w(forget);
   void *a = nullptr;
   {
-    Workspaces::Lease l = w.take(0, stream(1), 1000, 0, false);
+    Workspaces::Lease l = w.take(0, stream(1), 1000, 0);
     check(l && l.bytes == 1000, "a first buffer");
     a = l.p;
   }
-  check(w.take(0, stream(1), 500, 0, false).p == a, "a smaller request reuses it");
-  check(w.take(0, stream(2), 500, 0, false).p != a, "another stream has its own");
-  check(w.take(1, stream(1), 500, 0, false).p != a, "so has another device");
-  check(w.take(0, stream(1), 2000, 0, false).bytes == 2000, "a larger request");
+  check(w.take(0, stream(1), 500, 0).p == a, "a smaller request reuses it");
+  check(w.take(0, stream(2), 500, 0).p != a, "another stream has its own");
+  check(w.take(1, stream(1), 500, 0).p != a, "so has another device");
+  check(w.take(0, stream(1), 2000, 0).bytes == 2000, "a larger request");
   check(forgotten.count(a) == 1, "graphs that use the old buffer are dropped");
-  for (int i = 3; i < 40; ++i) w.take(0, stream(i), 1000 * i, 0, false);
+  for (int i = 3; i < 40; ++i) w.take(0, stream(i), 1000 * i, 0);
   check(syncs == 0, "growing buffers and many streams synchronize the device");
 }
 
@@ -100,15 +144,15 @@ static void reuse_and_growth() {
 static void out_of_memory() {
   Workspaces w(forget);
   const size_t before = limit;
-  check((bool)w.take(0, stream(1), 100, 0, false), "a small buffer");
+  check((bool)w.take(0, stream(1), 100, 0), "a small buffer");
   limit = used + 400;
-  check(w.take(0, stream(1), 1000, 300, false).bytes == 300, "no memory for a larger one: the smaller size");
+  check(w.take(0, stream(1), 1000, 300).bytes == 300, "no memory for a larger one: the smaller size");
   check(last_error == cudaSuccess, "a failed allocation leaves an error for the launch checks");
-  check(!w.take(0, stream(1), 2000, 1000, false), "no memory");
+  check(!w.take(0, stream(1), 2000, 1000), "no memory");
   limit = used;
-  check(!w.take(0, stream(2), 1, 0, false) && last_error == cudaSuccess, "no memory on a new stream");
+  check(!w.take(0, stream(2), 1, 0) && last_error == cudaSuccess, "no memory on a new stream");
   limit = before;
-  check(w.take(0, stream(2), 1, 0, false).bytes == 1, "a later call finds memory");
+  check(w.take(0, stream(2), 1, 0).bytes == 1, "a later call finds memory");
 }
 
 // Threads: while one holds a lease, its buffer is neither freed nor handed to
@@ -118,7 +162,7 @@ static void threads() {
   std::atomic<int> freed{0}, shared{0}, none{0};
   auto client = [&](int t, int s) {
     for (int i = 0; i < 200; ++i) {
-      Workspaces::Lease l = w.take(0, stream(s), 100 + 37 * ((i + t) % 5) * (1 + i / 20), 0, false);
+      Workspaces::Lease l = w.take(0, stream(s), 100 + 37 * ((i + t) % 5) * (1 + i / 20), 0);
       if (!l) {
         ++none;
         continue;
@@ -142,9 +186,61 @@ static void threads() {
   check(none == 0, "a stream found no memory");
 }
 
+// The graph of a capture and everything made from it are destroyed.
+static void destroy_graph(unsigned long long id) {
+  for (auto o : held[id]) cudaUserObjectRelease(o, 1);
+  held.erase(id);
+}
+
+// Stream captures: buffers of their own, that live as long as the graph.
+static void captures() {
+  Workspaces w(forget);
+  forgotten.clear();
+  void *own = w.take(0, stream(1), 1000, 0).p;
+  capturing[stream(1)] = 1;
+  void *a = w.take(0, stream(1), 1000, 0).p;
+  check(a && a != own, "a capture does not get the stream's buffer");
+  check(w.take(0, stream(1), 800, 0).p == a, "the next solve of that capture shares its buffer");
+  void *b = w.take(0, stream(1), 3000, 0).p;
+  check(b && b != a && live.count(a), "a larger one gets another, and the first stays");
+  capturing[stream(2)] = 1;  // forked in the same capture: runs beside it
+  void *c = w.take(0, stream(2), 1000, 0).p;
+  check(c && c != a && c != b, "two streams of one capture have their own");
+  capturing.clear();
+  capturing[stream(1)] = 2;
+  void *d = w.take(0, stream(1), 1000, 0).p;
+  check(d && d != a && d != own, "two captures on one stream have their own");
+  capturing.clear();
+  check(w.take(0, stream(1), 1000, 0).p == own, "outside the captures, the stream's own");
+  for (int i = 1; i < 30; ++i) w.take(0, stream(i), 100000, 0);
+  check(!live.count(own) && live.count(a) && live.count(b) && live.count(c) && live.count(d),
+        "larger solves and other streams leave the captures' buffers alone");
+  check(forgotten.count(a) + forgotten.count(b) + forgotten.count(c) + forgotten.count(d) == 0,
+        "the library's graphs have no part in them");
+  destroy_graph(1);
+  w.take(0, stream(1), 1, 0);
+  check(!live.count(a) && !live.count(b) && !live.count(c) && live.count(d), "gone with their graph");
+  destroy_graph(2);
+  w.take(0, stream(1), 1, 0);
+  check(!live.count(d), "and the last");
+  // no memory, or a graph that takes no objects: no buffer, none left behind
+  const size_t before = limit, was = used;
+  capturing[stream(3)] = 3;
+  limit = used;
+  check(!w.take(0, stream(3), 1000, 100), "no memory in a capture");
+  limit = before;
+  refuse_objects = true;
+  check(!w.take(0, stream(3), 1000, 100), "an object that the graph refuses");
+  refuse_objects = false;
+  check(used == was && last_error == cudaSuccess, "nothing is left of either");
+  capturing.clear();
+  check(syncs == 0, "captures synchronize");
+}
+
 int main() {
   reuse_and_growth();
   out_of_memory();
+  captures();
   threads();
   std::printf(fails ? "%d failed checks\n" : "ok\n", fails);
   return fails ? 1 : 0;

@@ -82,3 +82,109 @@ def test_threads_on_one_stream():
 
     in_threads([lambda k=k: worker(k) for k in range(len(sizes))])
     assert binding.device_error() == 0
+
+
+def captured(d, s, flags=0):
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        binding.apsp_fw(d, flags=flags, stream=s)
+    return g
+
+
+# aligned, unaligned, and int32 narrowed to int16 (sizes on both sides of the small-matrix schedule)
+@pytest.mark.parametrize("dt,n,ld,flags", [("i32", 512, 512, 0), ("f32", 512, 512, 0), ("i32", 2624, 2624, 0),
+                                           ("i32", 700, 701, 0), ("f32", 700, 701, 0),
+                                           ("i32", 512, 512, binding.FLAG_NARROW)])
+def test_capture_outlives_the_streams_workspace(dt, n, ld, flags):
+    # an ordinary call, a capture, then larger solves and other streams; the graph still solves
+    src = torch.zeros((n, ld), dtype=torch.int32 if dt == "i32" else torch.float32, device="cuda")
+    w = graph(dt, n, n)
+    if flags:  # (n - 1) Wmax < 16383
+        w = torch.where(w < inputs.INF_I32, w.clamp(max=30), w)
+    src[:, :n] = w
+    d = src.clone()
+    ref = src.clone()
+    binding.apsp_fw(ref, n, flags=binding.FLAG_NO_WORKSPACE | binding.FLAG_NO_GRAPH)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        binding.apsp_fw(d, n, flags=flags, stream=s)
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        binding.apsp_fw(d, n, flags=flags, stream=s)
+    big = graph(dt, n + 1500, 1)
+    others = [s] + [torch.cuda.Stream() for _ in range(18)]
+    for t in others:
+        with torch.cuda.stream(t):
+            x = big.clone()
+            x.record_stream(t)
+            binding.apsp_fw(x, stream=t)
+    torch.cuda.synchronize()
+    del x
+    torch.cuda.empty_cache()
+    junk = torch.full((1 << 27,), 123456789, dtype=torch.int32, device="cuda")  # over what was freed
+    for _ in range(2):
+        d.copy_(src)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(d, ref)
+    assert bool((junk == 123456789).all())
+    assert binding.device_error() == 0
+
+
+@pytest.mark.parametrize("dt,n", [("i32", 900), ("f32", 900), ("i32", 2624)])
+def test_two_graphs_of_one_stream_side_by_side(dt, n):
+    srcs = [graph(dt, n, n + k) for k in range(2)]
+    refs = [solved(x) for x in srcs]
+    ds = [torch.empty_like(x) for x in srcs]
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        ds[0].copy_(srcs[0])
+        binding.apsp_fw(ds[0], stream=s)
+    s.synchronize()
+    gs = [captured(d, s) for d in ds]
+    ts = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for _ in range(10):
+        for k in range(2):
+            with torch.cuda.stream(ts[k]):
+                ds[k].copy_(srcs[k])
+                gs[k].replay()
+        torch.cuda.synchronize()
+        for k in range(2):
+            assert torch.equal(ds[k], refs[k])
+
+
+def test_first_call_of_a_stream_in_a_capture():
+    for dt, n in (("i32", 1000), ("f32", 3500), ("i32", 2624)):
+        src = graph(dt, n, n)
+        ref = solved(src)
+        d = src.clone()
+        s = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        g = captured(d, s)
+        d.copy_(src)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(d, ref)
+
+
+def test_graphs_give_their_workspaces_back():
+    n = 3300  # 52 stages: 3.4 MB each
+    d = graph("f32", n, 3)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def cycle(count):
+        for _ in range(count):
+            captured(d, s).reset()
+        binding.apsp_fw(d, stream=s)
+        torch.cuda.synchronize()
+
+    cycle(5)
+    torch.cuda.empty_cache()
+    free0 = torch.cuda.mem_get_info()[0]
+    cycle(100)
+    torch.cuda.empty_cache()
+    assert torch.cuda.mem_get_info()[0] > free0 - (150 << 20)
