@@ -40,6 +40,8 @@
  * general: the output is then unspecified (the paper excludes it).
  *
  * Threading: all entry points are reentrant for distinct matrices.
+ * cudaStreamPerThread is a stream of its own in every thread; a thread that
+ * solves on it waits for that work before it ends.
  */
 #ifndef APSP_H
 #define APSP_H
@@ -188,8 +190,8 @@ APSP_API int apsp_version(void);
  * Other layouts: below 22 stages of s = 64 the kernels take any layout; from
  * there on the matrix is solved on an aligned copy (n x n elements of
  * device memory in stream order for the duration of the solve, from a pool of
- * the library that keeps at most 64 MiB); without memory for it, or while the
- * stream is being captured, it is solved in place (same results, slower: the
+ * the library that keeps at most 64 MiB); without memory for it, while the
+ * stream is being captured, or on cudaStreamPerThread, it is solved in place (same results, slower: the
  * kernels for any layout up to the stage counts of apsp_config.lookahead, a
  * generic kernel above).
  * Returns APSP_EINVAL on a bad argument, APSP_ECUDA if a launch fails.

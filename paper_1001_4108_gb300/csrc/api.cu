@@ -92,9 +92,12 @@ int run_dtype(const RunArgs &a, int dtype) {
 // capture.  Work on one launching stream is ordered, so its solves can share
 // them; a wait always refers to a record enqueued before it, so calls from
 // several threads on one stream can only over-synchronise, never deadlock.
+// cudaStreamPerThread is another stream in every thread: `id` tells them
+// apart (0 for other handles).
 struct SideEntry {
   int dev;
   cudaStream_t stream;
+  unsigned long long id;
   cudaStream_t side;
   cudaEvent_t fork, join;
   int prio;
@@ -106,8 +109,13 @@ std::vector<SideEntry> g_side;
 // holds g_mu.
 void side_resources_locked(int dev, cudaStream_t stream, bool capturing, RunArgs *a) {
   a->side = nullptr;
+  unsigned long long id = 0;
+  if (stream == cudaStreamPerThread && cudaStreamGetId(stream, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
   for (auto &e : g_side)
-    if (e.dev == dev && e.stream == stream) {
+    if (e.dev == dev && e.stream == stream && e.id == id) {
       a->side = e.side;
       a->fork = e.fork;
       a->join = e.join;
@@ -119,7 +127,7 @@ void side_resources_locked(int dev, cudaStream_t stream, bool capturing, RunArgs
   if (capturing || g_side.size() >= kMaxSide) return;
   int least = 0, greatest = 0;
   if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess) return;
-  SideEntry e{dev, stream, nullptr, nullptr, nullptr, greatest};
+  SideEntry e{dev, stream, id, nullptr, nullptr, nullptr, greatest};
   if (cudaStreamCreateWithPriority(&e.side, cudaStreamNonBlocking, greatest) != cudaSuccess) return;
   if (cudaEventCreateWithFlags(&e.fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&e.join, cudaEventDisableTiming) != cudaSuccess) {
@@ -424,7 +432,8 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   const bool any_layout = stage_need && a.ws_bytes >= stage_need && R < kStageCopyRounds;
   void *copy = nullptr;
   const int64_t cld = (n * (int64_t)es + 15) / 16 * 16 / (int64_t)es;
-  if (!a.tma_ok && !any_layout && R > 1 && !(a.flags & kInPlace) && cap == cudaStreamCaptureStatusNone)
+  if (!a.tma_ok && !any_layout && R > 1 && !(a.flags & kInPlace) && cap == cudaStreamCaptureStatusNone &&
+      a.stream != cudaStreamPerThread)  // see Workspaces::take
     copy = g_copies.alloc(dev, (size_t)n * cld * es, a.stream);
   if (copy) {
     if (copy_matrix(dist, ld, copy, cld, n, (int)es, a.stream) != APSP_OK) st = APSP_ECUDA;

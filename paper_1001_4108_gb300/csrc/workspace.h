@@ -8,6 +8,7 @@
 // object; once the last of them is gone the memory goes back to the pool.
 #pragma once
 
+#include <algorithm>
 #include <atomic>
 #include <cstddef>
 #include <memory>
@@ -69,12 +70,14 @@ class StreamPool {
 class Workspaces {
   struct Entry {
     int dev;
-    cudaStream_t stream;
-    std::mutex mu;  // held from take() until the work that uses the buffer is enqueued
+    unsigned long long id = 0;  // the stream's
+    std::mutex mu;              // held from take() until the work that uses the buffer is enqueued
     void *p = nullptr;
     size_t bytes = 0;
-    unsigned long long capture = 0;  // the capture whose graph holds the buffer
-    std::atomic<bool> unused{false}; // that graph and its offspring are gone
+    // buffers of captures: the stream's handle, the capture whose graph holds the buffer
+    cudaStream_t stream = nullptr;
+    unsigned long long capture = 0;
+    std::atomic<bool> unused{false};  // that graph and its offspring are gone
   };
 
  public:
@@ -123,6 +126,9 @@ class Workspaces {
   // At least `bytes` bytes for work on `stream`, else at least `least` (if not
   // 0), else an empty lease: there is no memory.  The caller then runs kernels
   // that need less or none.
+  // Nothing is allocated or freed in the order of cudaStreamPerThread, which
+  // ends with its thread: a thread that ended with such frees pending left a
+  // later device synchronize waiting.
   Lease take(int dev, cudaStream_t stream, size_t bytes, size_t least) {
     Lease l;
     l.stream_ = stream;
@@ -140,37 +146,46 @@ class Workspaces {
             capturing ? captured(dev, stream, capture, graph, bytes, least) : entry(dev, stream)) {
       l.lk_ = std::unique_lock<std::mutex>(e->mu);
       if (e->bytes < bytes && !capturing) {
-        // in stream order: all work that uses the buffer is on this stream
-        if (e->p) {
-          forget_(e->p, e->bytes);
-          cudaFreeAsync(e->p, stream);
+        if (e->p) forget_(e->p, e->bytes);
+        if (stream == cudaStreamPerThread) {
+          replace_outside(e.get(), bytes, least);
+        } else {  // in stream order: all work that uses the buffer is on this stream
+          if (e->p) cudaFreeAsync(e->p, stream);
+          e->bytes = alloc(pool_, dev, stream, bytes, least, &e->p);
         }
-        e->bytes = alloc(dev, stream, bytes, least, &e->p);
       }
-      if (e->p) {
+      if (e->p && e->bytes >= (least ? std::min(bytes, least) : bytes)) {
         l.p = e->p;
         l.bytes = e->bytes;
         l.entry_ = e;
       } else {
         l.lk_.unlock();
       }
-    } else if (!capturing) {
-      l.bytes = alloc(dev, stream, bytes, least, &l.p);  // more streams than entries: a buffer for this call
+    } else if (!capturing && stream != cudaStreamPerThread) {
+      l.bytes = alloc(pool_, dev, stream, bytes, least, &l.p);  // more streams than entries: for this call
     }
     return l;
   }
 
  private:
   static constexpr size_t kMaxEntries = 16;
-  // Entries are never evicted: another stream's work may be using the buffer.
+  // By the stream's id, not its handle: every thread's cudaStreamPerThread is
+  // another stream, and a destroyed stream's handle can come back while its
+  // work still runs.  Entries are never evicted: another stream's work may be
+  // using the buffer.
   std::shared_ptr<Entry> entry(int dev, cudaStream_t stream) {
+    unsigned long long id = 0;
+    if (cudaStreamGetId(stream, &id) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
     std::lock_guard<std::mutex> lk(mu_);
     for (auto &e : entries_)
-      if (e->dev == dev && e->stream == stream) return e;
+      if (e->dev == dev && e->id == id) return e;
     if (entries_.size() >= kMaxEntries) return nullptr;
     auto e = std::make_shared<Entry>();
     e->dev = dev;
-    e->stream = stream;
+    e->id = id;
     entries_.push_back(e);
     return e;
   }
@@ -188,9 +203,7 @@ class Workspaces {
     e->dev = dev;
     e->stream = stream;
     e->capture = capture;
-    for (const size_t want : {bytes, least})
-      if (!e->p && want && (e->p = capture_pool_.alloc(dev, want, home))) e->bytes = want;
-    if (!e->p) return nullptr;
+    if (!(e->bytes = alloc(outside_, dev, home, bytes, least, &e->p))) return nullptr;
     auto *held = new std::shared_ptr<Entry>(e);
     cudaUserObject_t object = nullptr;
     const bool made =
@@ -207,39 +220,50 @@ class Workspaces {
     captured_.push_back(e);
     return e;
   }
+  // A larger buffer for a calling thread's own stream; it waits for that
+  // stream's work with the old one.
+  void replace_outside(Entry *e, size_t bytes, size_t least) {
+    if (e->p && cudaStreamSynchronize(cudaStreamPerThread) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lk(mu_);
+    const cudaStream_t home = home_stream(e->dev);
+    if (!home) return;
+    if (e->p) cudaFreeAsync(e->p, home);
+    e->bytes = alloc(outside_, e->dev, home, bytes, least, &e->p);
+    cudaStreamSynchronize(home);
+  }
   // Runs on a thread of the CUDA runtime when nothing refers to a capture's
   // graph any more: no CUDA calls in here.
   static void CUDART_CB graph_gone(void *held) {
     auto *e = static_cast<std::shared_ptr<Entry> *>(held);
     (*e)->unused = true;
-    ++unused_;
+    unused_ = true;
     delete e;
   }
   // Returns the buffers of captures that are gone to their pool.
   void give_back(int dev) {
-    if (unused_ == 0) return;
+    if (!unused_ || !unused_.exchange(false)) return;
     const OutsideCapture guard;
     std::lock_guard<std::mutex> lk(mu_);
     for (size_t i = 0; i < captured_.size();) {
       if (captured_[i]->unused && captured_[i]->dev == dev) {
         cudaFreeAsync(captured_[i]->p, home_[dev]);
         captured_.erase(captured_.begin() + i);
-        --unused_;
       } else {
+        if (captured_[i]->unused) unused_ = true;  // for a call on its device
         ++i;
       }
     }
   }
-  // The stream of the captures' allocations: nothing else runs on it.
+  // The stream of the allocations outside_: nothing else runs on it.
   cudaStream_t home_stream(int dev) {
     if (!home_[dev] && !got_memory(cudaStreamCreateWithFlags(&home_[dev], cudaStreamNonBlocking)))
       home_[dev] = nullptr;
     return home_[dev];
   }
   // `bytes` or else `least` bytes in *p; the size, 0 (*p = nullptr) without memory
-  size_t alloc(int dev, cudaStream_t stream, size_t bytes, size_t least, void **p) {
+  static size_t alloc(StreamPool &pool, int dev, cudaStream_t stream, size_t bytes, size_t least, void **p) {
     for (const size_t want : {bytes, least})
-      if (want && (*p = pool_.alloc(dev, want, stream))) return want;
+      if (want && (*p = pool.alloc(dev, want, stream))) return want;
     *p = nullptr;
     return 0;
   }
@@ -248,8 +272,8 @@ class Workspaces {
   std::vector<std::shared_ptr<Entry>> entries_;
   StreamPool pool_{64ull << 20};
   std::vector<std::shared_ptr<Entry>> captured_;
-  static inline std::atomic<int> unused_{0};  // entries of captured_ whose graph is gone
-  StreamPool capture_pool_{64ull << 20};
+  static inline std::atomic<bool> unused_{false};  // some entry of captured_ may be unused
+  StreamPool outside_{64ull << 20};  // buffers that no stream's order covers
   cudaStream_t home_[kMaxDev] = {};
 };
 

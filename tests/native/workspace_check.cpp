@@ -26,6 +26,8 @@ std::set<void *> forgotten, leased;
 std::map<cudaStream_t, unsigned long long> capturing;            // stream -> capture, also its graph
 std::map<unsigned long long, std::vector<cudaUserObject_t>> held;  // graph -> its objects
 bool refuse_objects = false;
+std::atomic<int> thread_count{0}, per_thread_order{0};
+std::map<cudaStream_t, int> recreated;  // how often a handle was destroyed and handed out again
 
 cudaError_t take(void **p, size_t bytes) {
   std::lock_guard<std::mutex> lk(mu);
@@ -74,8 +76,14 @@ cudaError_t cudaMemPoolCreate(cudaMemPool_t *pool, const cudaMemPoolProps *) {
   return cudaSuccess;
 }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
-cudaError_t cudaMallocFromPoolAsync(void **p, size_t bytes, cudaMemPool_t, cudaStream_t) { return take(p, bytes); }
-cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return give(p); }
+cudaError_t cudaMallocFromPoolAsync(void **p, size_t bytes, cudaMemPool_t, cudaStream_t s) {
+  if (s == cudaStreamPerThread) ++per_thread_order;
+  return take(p, bytes);
+}
+cudaError_t cudaFreeAsync(void *p, cudaStream_t s) {
+  if (s == cudaStreamPerThread) ++per_thread_order;
+  return give(p);
+}
 cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *mode) {
   thread_local cudaStreamCaptureMode current = cudaStreamCaptureModeGlobal;
   std::swap(*mode, current);
@@ -86,7 +94,7 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
   return cudaSuccess;
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
-  if (s != stream(99)) ++syncs;
+  if (s != stream(99) && s != cudaStreamPerThread) ++syncs;
   return cudaSuccess;
 }
 cudaError_t cudaStreamGetCaptureInfo(cudaStream_t s, cudaStreamCaptureStatus *status, unsigned long long *id,
@@ -99,6 +107,11 @@ cudaError_t cudaStreamGetCaptureInfo(cudaStream_t s, cudaStreamCaptureStatus *st
     *id = it->second;
     *graph = reinterpret_cast<cudaGraph_t>((uintptr_t)it->second);
   }
+  return cudaSuccess;
+}
+cudaError_t cudaStreamGetId(cudaStream_t s, unsigned long long *id) {
+  thread_local const unsigned long long mine = 1000 + thread_count++;
+  *id = s == cudaStreamPerThread ? mine : reinterpret_cast<uintptr_t>(s) + recreated[s];
   return cudaSuccess;
 }
 cudaError_t cudaUserObjectCreate(cudaUserObject_t *o, void *p, cudaHostFn_t destroy, unsigned, unsigned) {
@@ -153,6 +166,23 @@ static void out_of_memory() {
   check(!w.take(0, stream(2), 1, 0) && last_error == cudaSuccess, "no memory on a new stream");
   limit = before;
   check(w.take(0, stream(2), 1, 0).bytes == 1, "a later call finds memory");
+}
+
+// One handle, several streams: each has its own buffer.
+static void stream_identity() {
+  Workspaces w(forget);
+  Workspaces::Lease mine = w.take(0, cudaStreamPerThread, 1000, 0);
+  void *other = nullptr;
+  std::thread([&] { other = w.take(0, cudaStreamPerThread, 1000, 0).p; }).join();
+  check(mine && other && other != mine.p, "two threads' cudaStreamPerThread share a buffer");
+  mine.release();
+  check(w.take(0, cudaStreamPerThread, 5000, 0).bytes == 5000, "and can grow");
+  for (int i = 0; i < 20; ++i) std::thread([&] { w.take(0, cudaStreamPerThread, 1000, 0); }).join();
+  check(per_thread_order == 0, "memory in the order of a thread's own stream");
+  Workspaces v(forget);
+  void *a = v.take(0, stream(1), 1000, 0).p;
+  ++recreated[stream(1)];
+  check(v.take(0, stream(1), 1000, 0).p != a, "a new stream has the buffer of a destroyed one of that handle");
 }
 
 // Threads: while one holds a lease, its buffer is neither freed nor handed to
@@ -241,6 +271,7 @@ int main() {
   reuse_and_growth();
   out_of_memory();
   captures();
+  stream_identity();
   threads();
   std::printf(fails ? "%d failed checks\n" : "ok\n", fails);
   return fails ? 1 : 0;

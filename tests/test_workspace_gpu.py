@@ -1,5 +1,6 @@
 """Lifetime and sharing of the library's own workspaces: solves from many
 threads and streams at once, each compared with its plain result."""
+import ctypes
 import threading
 
 import pytest
@@ -188,3 +189,30 @@ def test_graphs_give_their_workspaces_back():
     cycle(100)
     torch.cuda.empty_cache()
     assert torch.cuda.mem_get_info()[0] > free0 - (150 << 20)
+
+
+def test_per_thread_default_streams():
+    # the handle cudaStreamPerThread (2) from four threads at once: four streams
+    # (each waits for its solves before it ends)
+    per_thread = 2
+    rt = ctypes.CDLL("libcudart.so." + torch.version.cuda.split(".")[0])
+    n = 1100
+    srcs = [graph("i32" if k % 2 else "f32", n, n + k) for k in range(4)]
+    refs = [solved(x) for x in srcs]
+    ds = [[x.clone() for _ in range(6)] for x in srcs]
+    torch.cuda.synchronize()
+    code = [binding.APSP_F32, binding.APSP_I32]
+
+    def worker(k):
+        opt = binding.Options(0, binding.FLAG_NO_GRAPH, None, 0, None, 0)
+        try:
+            for d in ds[k]:
+                assert binding.apsp_fw_raw(d.data_ptr(), n, n, code[k % 2], per_thread, opt) == binding.APSP_OK
+        finally:
+            assert rt.cudaStreamSynchronize(ctypes.c_void_p(per_thread)) == 0
+
+    in_threads([lambda k=k: worker(k) for k in range(4)])
+    torch.cuda.synchronize()
+    for k in range(4):
+        for d in ds[k]:
+            assert torch.equal(d, refs[k]), k
