@@ -215,21 +215,6 @@ void forget_graphs_using(void *p, size_t bytes) {
 
 Workspaces g_workspaces(forget_graphs_using);
 
-// One panel copy (fp32 interleaved row panel, int16 replicated column panel).
-size_t panel_bytes_for(int64_t n, int dtype, int S) {
-  if (n <= S) return 0;
-  if (dtype == APSP_F32) return interleaved_panel_bytes(n, S);
-  if (dtype == APSP_I16) return replicated_panel_bytes(n, S);
-  return 0;
-}
-
-// One panel buffer, two when the lookahead schedule applies (phase 2 of the
-// next stage writes its copy while phase 3 reads the current one).
-size_t workspace_bytes_for(int64_t n, int dtype, int S) {
-  const size_t bufs = (n + S - 1) / S >= kLookaheadMinRounds ? 2 : 1;
-  return bufs * panel_bytes_for(n, dtype, S);
-}
-
 // The workspace a call with `flags` uses: with APSP_FLAG_ONE_LAUNCH on a
 // small matrix, at least the one-launch schedule's per-tile flags.
 size_t workspace_bytes_with(int64_t n, int dtype, int S, int flags) {
@@ -299,10 +284,12 @@ extern "C" int apsp_query_config(int64_t n, int dtype, int32_t kblock, apsp_conf
 
 namespace apsp {
 namespace {
-// apsp_fw_ex, optionally with the path bookkeeping of apsp_fw_paths.
+// apsp_fw_ex, optionally with the path bookkeeping of apsp_fw_paths, with host
+// memory for the first and last stage's tiles, with the library's part of the
+// memory supplied (scratch).
 int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt, void *stream, int16_t *via,
           int64_t via_ld, const void *first_src = nullptr, int64_t first_src_ld = 0, void *last_dst = nullptr,
-          int64_t last_dst_ld = 0) {
+          int64_t last_dst_ld = 0, void *scratch = nullptr, size_t scratch_bytes = 0) {
   int st = check_args(dist, n, ld, dtype, opt);
   if (st != APSP_OK) return st;
   if (n == 0) return APSP_OK;
@@ -382,18 +369,13 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   }
   const size_t need = (a.flags & APSP_FLAG_NO_WORKSPACE) ? 0 : workspace_bytes_with(n, dtype, a.S, a.flags);
   const int R = (int)((n + a.S - 1) / a.S);
-  const size_t stage_need =
-      uses_stage_launches(a.S, R, dtype, via != nullptr, a.flags, a.events != nullptr)
-          ? stage_ws_bytes(R, dtype == APSP_I16)
-          : 0;
-  // the int32 kernels that read both panels from copies, not the matrix
-  constexpr int kNoPairs = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_WORKSPACE;
-  const size_t pairs_need = stage_need || dtype != APSP_I32 || R < 2 || (a.flags & kNoPairs)
-                                ? 0
-                                : (R >= kLookaheadMinRounds ? 4 : 2) * interleaved_panel_bytes(n, a.S);
-  const size_t more = std::max(stage_need, pairs_need);
+  const bool staged = uses_stage_launches(a.S, R, dtype, via != nullptr, a.flags, a.events != nullptr);
+  const size_t more = fast_workspace_bytes(n, dtype, a.S, via != nullptr, a.flags, a.events != nullptr);
   Workspaces::Lease lease;  // until everything is enqueued
-  if (need || more) {
+  if (scratch) {
+    a.ws = scratch;
+    a.ws_bytes = scratch_bytes;
+  } else if (need || more) {
     if (opt && opt->workspace && !need) {
       // not asked for: taken if it is enough for the kernels that can use one
       a.ws = opt->workspace;
@@ -429,7 +411,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   // 1025 255 and 266, 1537 487 and 442, 2047 775 and 641.
   constexpr int kStageCopyRounds = 22;
   constexpr int kInPlace = APSP_FLAG_GENERIC | APSP_FLAG_NO_WORKSPACE;
-  const bool any_layout = stage_need && a.ws_bytes >= stage_need && R < kStageCopyRounds;
+  const bool any_layout = staged && a.ws_bytes >= more && R < kStageCopyRounds;
   void *copy = nullptr;
   const int64_t cld = (n * (int64_t)es + 15) / 16 * 16 / (int64_t)es;
   if (!a.tma_ok && !any_layout && R > 1 && !(a.flags & kInPlace) && cap == cudaStreamCaptureStatusNone &&
@@ -452,6 +434,14 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   return APSP_OK;
 }
 }  // namespace
+
+int solve_request(void *dist, int64_t n, int64_t ld, int dtype, int kblock, void *scratch, size_t scratch_bytes,
+                  cudaStream_t stream) {
+  apsp_options o{};
+  o.kblock = kblock;
+  o.flags = APSP_FLAG_NO_GRAPH;  // device addresses change from request to request
+  return solve(dist, n, ld, dtype, &o, stream, nullptr, 0, nullptr, 0, nullptr, 0, scratch, scratch_bytes);
+}
 }  // namespace apsp
 
 extern "C" int apsp_fw_ex(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt, void *stream) {

@@ -2,6 +2,7 @@
 // per-element-type translation units (fw_i32.cu, fw_f32.cu, fw_i16.cu).
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -131,6 +132,47 @@ inline size_t interleaved_panel_bytes(int64_t n, int S) {
   return (size_t)S * (size_t)np * sizeof(float);
 }
 
+// One panel copy (fp32 interleaved row panel, int16 replicated column panel).
+inline size_t panel_bytes_for(int64_t n, int dtype, int S) {
+  if (n <= S) return 0;
+  if (dtype == APSP_F32) return interleaved_panel_bytes(n, S);
+  if (dtype == APSP_I16) return replicated_panel_bytes(n, S);
+  return 0;
+}
+
+// One panel buffer, two when the lookahead schedule applies (phase 2 of the
+// next stage writes its copy while phase 3 reads the current one).
+inline size_t workspace_bytes_for(int64_t n, int dtype, int S) {
+  const size_t bufs = (n + S - 1) / S >= kLookaheadMinRounds ? 2 : 1;
+  return bufs * panel_bytes_for(n, dtype, S);
+}
+
+// What the library allocates beyond that for the faster forms: the panels and
+// diagonal tiles of stage.cuh, or both panels of an int32 solve in copies (two
+// of each for the lookahead schedule).  0: there is no such form.
+inline size_t fast_workspace_bytes(int64_t n, int dtype, int S, bool via, int flags, bool traced) {
+  constexpr int kNoPairs = APSP_FLAG_GENERIC | APSP_FLAG_REVERSE_K | APSP_FLAG_NO_WORKSPACE;
+  const int R = (int)((n + S - 1) / S);
+  if (uses_stage_launches(S, R, dtype, via, flags, traced)) return stage_ws_bytes(R, dtype == APSP_I16);
+  if (dtype != APSP_I32 || R < 2 || (flags & kNoPairs)) return 0;
+  return (R >= kLookaheadMinRounds ? 4 : 2) * interleaved_panel_bytes(n, S);
+}
+
+// The most that a solve of up to max_n vertices without special requests uses,
+// in any element type and with either tile side.
+inline size_t request_workspace_bytes(int64_t max_n) {
+  size_t bytes = 0;
+  for (const int dtype : {APSP_I32, APSP_F32, APSP_I16})
+    for (const int S : {64, 128}) {
+      const int64_t staged = (int64_t)stage_max_rounds(dtype == APSP_F32, dtype == APSP_I16, false) * S;
+      for (const int64_t n : {max_n, std::min(max_n, staged)}) {
+        const size_t a = workspace_bytes_for(n, dtype, S), b = fast_workspace_bytes(n, dtype, S, false, 0, false);
+        bytes = std::max(bytes, std::max(a, b));
+      }
+    }
+  return bytes;
+}
+
 // One graph of a batch (device matrix, leading dimension, vertices).
 struct BatchDesc {
   void *d;
@@ -170,6 +212,11 @@ int check_negcycle(void *dist, int64_t n, int64_t ld, int dtype, cudaStream_t st
 int narrow_to_i16(const int32_t *src, int64_t n, int64_t ld, int16_t *dst, int64_t ld16, cudaStream_t st);
 int copy_matrix(const void *src, int64_t sld, void *dst, int64_t dld, int64_t n, int elem, cudaStream_t st);
 int widen_from_i16(const int16_t *src, int64_t ld16, int64_t n, int32_t *dst, int64_t ld, cudaStream_t st);
+
+// apsp_fw_ex without the graph cache on scratch memory of the caller
+// (request_workspace_bytes, 256-byte aligned): the schedule of an apsp_fw call.
+int solve_request(void *dist, int64_t n, int64_t ld, int dtype, int kblock, void *scratch, size_t scratch_bytes,
+                  cudaStream_t stream);
 
 // Tile side the C ABI picks for (n, dtype) when none is requested.
 int default_kblock(int64_t n, int dtype);

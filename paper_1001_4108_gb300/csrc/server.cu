@@ -155,8 +155,8 @@ struct Server {
   int64_t bytes_resident = 0;
   int inflight = 0;
   std::vector<cudaStream_t> streams;  // [0]: batched launches; the rest: one large request each, round robin
-  std::vector<void *> workspaces;     // per stream, for apsp_fw_ex
-  int64_t ws_bytes = 0;
+  std::vector<void *> workspaces;     // per stream, for solve_request
+  size_t ws_bytes = 0;
   size_t next_stream = 1;
   std::vector<double> lat_ms;
   int64_t submitted = 0, completed = 0, failed = 0;
@@ -235,12 +235,9 @@ void launch_admitted(Server *s, std::vector<Request *> &adm) {
     if (rc == APSP_OK && cudaMemcpyAsync(r->dev, r->host, r->bytes, cudaMemcpyHostToDevice, st) != cudaSuccess)
       rc = APSP_ECUDA;
     if (rc == APSP_OK) {
-      apsp_options o{};
-      o.flags = APSP_FLAG_NO_GRAPH;  // device addresses change from request to request
-      if (r->n <= kBatchCtaMaxN) o.kblock = 64;  // the batched kernels' depth: same result either way
-      o.workspace = s->workspaces[si];
-      o.workspace_bytes = s->ws_bytes;
-      rc = apsp_fw_ex(r->dev, r->n, r->ld, r->dtype, &o, st);
+      // up to the batched kernels' limit their depth: same result either way
+      rc = solve_request(r->dev, r->n, r->ld, r->dtype, r->n <= kBatchCtaMaxN ? 64 : 0, s->workspaces[si], s->ws_bytes,
+                         st);
     }
     if (rc == APSP_OK && cudaMemcpyAsync(r->host, r->dev, r->bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess)
       rc = APSP_ECUDA;
@@ -395,12 +392,17 @@ extern "C" int apsp_server_create(apsp_server **out, const apsp_server_config *c
   cudaSetDevice(cfg->device);
   int rc = APSP_OK;
   const int nstreams = 1 + std::max(1, cfg->streams ? cfg->streams : 4);
-  s->ws_bytes = std::max(apsp_workspace_bytes(cfg->max_n, APSP_F32, 0), apsp_workspace_bytes(cfg->max_n, APSP_I16, 0));
+  // Enough for any request to take the schedule that apsp_fw takes for its size
+  // and type, whatever max_n is.  Bursts, ms, with this and with the lookahead
+  // schedule for all: 48 requests of n log-uniform in 32..2048 5.65 and 6.4,
+  // another 48 4.7 and 4.8, 24 of 600..3000 10.8 and 11.0, 40 of 520..1500 7.0
+  // and 6.9, 8 of 1500..3000 10.05 and 11.1.
+  s->ws_bytes = request_workspace_bytes(cfg->max_n);
   for (int i = 0; i < nstreams && rc == APSP_OK; ++i) {
     cudaStream_t st = nullptr;
     void *ws = nullptr;
     if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) rc = APSP_ECUDA;
-    if (rc == APSP_OK && s->ws_bytes && !got_memory(cudaMalloc(&ws, (size_t)s->ws_bytes))) rc = APSP_ENOMEM;
+    if (rc == APSP_OK && s->ws_bytes && !got_memory(cudaMalloc(&ws, s->ws_bytes))) rc = APSP_ENOMEM;
     s->streams.push_back(st);
     s->workspaces.push_back(ws);
   }

@@ -267,7 +267,22 @@ static void captures() {
   check(syncs == 0, "captures synchronize");
 }
 
+// A server's workspaces: a request's schedule does not depend on max_n.
+static void request_sizes() {
+  bool enough = true;
+  for (const int64_t max_n : {1, 64, 65, 512, 1984, 2048, 2496, 3328, 3329, 4096, 6000, 16384})
+    for (int64_t n = 1; n <= max_n; n += n < 200 ? 1 : 61)
+      for (const int dtype : {APSP_I32, APSP_F32, APSP_I16})
+        for (const int S : {64, 128}) {
+          const size_t have = apsp::request_workspace_bytes(max_n);
+          enough = enough && have >= apsp::workspace_bytes_for(n, dtype, S) &&
+                   have >= apsp::fast_workspace_bytes(n, dtype, S, false, APSP_FLAG_NO_GRAPH, false);
+        }
+  check(enough, "a request has less memory than its schedule needs");
+}
+
 int main() {
+  request_sizes();
   reuse_and_growth();
   out_of_memory();
   captures();

@@ -216,3 +216,15 @@ def test_per_thread_default_streams():
     for k in range(4):
         for d in ds[k]:
             assert torch.equal(d, refs[k]), k
+
+
+def test_server_requests_on_both_sides_of_the_schedules():
+    # 31, 32, 39 and 41 stages (int32 panel copies beyond 39), whatever the largest size of the server
+    sizes = [1984, 1985, 2496, 2560]
+    for max_n in (2560, 4096):
+        with binding.Server(max_inflight=8, hbm_budget_bytes=1 << 30, max_n=max_n) as server:
+            srcs = [graph(dt, n, n) for n in sizes for dt in ("i32", "f32")]
+            tickets = [server.submit(x) for x in srcs]
+            for x, t in zip(srcs, tickets):
+                assert torch.equal(torch.from_numpy(server.wait(t)), solved(x).cpu()), x.shape
+    assert binding.device_error() == 0
