@@ -140,7 +140,8 @@ typedef struct apsp_options {
        bytes (at least one panel buffer, half of that from 3 stages on: then
        the plain schedule runs), 256-byte aligned, owned by the caller and used
        only between the enqueue and the completion of this call's work on its
-       stream; smaller: APSP_EINVAL.
+       stream; smaller: APSP_EINVAL.  Left alone where that is 0 (int32, but
+       for APSP_FLAG_ONE_LAUNCH's flags).
        NULL = the library uses a buffer of its own, one per (device, stream),
        allocated on first use.  A solve in a stream capture gets a buffer that
        belongs to the captured graph (shared by the solves captured on one

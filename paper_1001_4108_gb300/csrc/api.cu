@@ -375,23 +375,22 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   if (scratch) {
     a.ws = scratch;
     a.ws_bytes = scratch_bytes;
-  } else if (need || more) {
-    if (opt && opt->workspace && !need) {
-      // not asked for: taken if it is enough for the kernels that can use one
-      a.ws = opt->workspace;
-      a.ws_bytes = (size_t)std::max<int64_t>(opt->workspace_bytes, 0);
-    } else if (opt && opt->workspace) {
-      // one panel buffer is enough (plain schedule); two allow the lookahead
+  } else if (opt && opt->workspace) {
+    // one panel buffer is enough (plain schedule); two allow the lookahead.
+    // Where apsp_workspace_bytes asks for nothing (int32) what the caller has
+    // there is left alone, but for the flags of APSP_FLAG_ONE_LAUNCH.
+    if (need) {
       if (opt->workspace_bytes < (int64_t)panel_bytes_for(n, dtype, a.S) ||
           reinterpret_cast<uintptr_t>(opt->workspace) % 256)
         return APSP_EINVAL;
       a.ws = opt->workspace;
       a.ws_bytes = (size_t)opt->workspace_bytes;
-    } else {
-      lease = g_workspaces.take(dev, a.stream, std::max(need, more), need);
-      a.ws = lease.p;  // none: the kernels fall back to the form that needs none
-      a.ws_bytes = lease.bytes;
+      if (dtype == APSP_I32) a.ws_bytes = std::min(a.ws_bytes, need);
     }
+  } else if (need || more) {
+    lease = g_workspaces.take(dev, a.stream, std::max(need, more), need);
+    a.ws = lease.p;  // none: the kernels fall back to the form that needs none
+    a.ws_bytes = lease.bytes;
   }
   if (!(a.flags & APSP_FLAG_NO_LOOKAHEAD)) {
     std::lock_guard<std::mutex> lk(g_mu);

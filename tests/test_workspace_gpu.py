@@ -228,3 +228,22 @@ def test_server_requests_on_both_sides_of_the_schedules():
             for x, t in zip(srcs, tickets):
                 assert torch.equal(torch.from_numpy(server.wait(t)), solved(x).cpu()), x.shape
     assert binding.device_error() == 0
+
+
+@pytest.mark.parametrize("n,ld,offset", [(700, 704, 0), (700, 701, 0), (2624, 2624, 0), (1500, 1501, 1)])
+def test_int32_leaves_a_callers_workspace_alone(n, ld, offset):
+    # apsp_workspace_bytes asks for none: neither written nor refused, aligned or not
+    assert binding.workspace_bytes(n, binding.APSP_I32) == 0
+    src = torch.zeros((n, ld), dtype=torch.int32, device="cuda")
+    src[:, :n] = graph("i32", n, n)
+    ref = src.clone()
+    binding.apsp_fw(ref, n, flags=binding.FLAG_NO_WORKSPACE)
+    ws = torch.full((6 << 20,), 77, dtype=torch.int32, device="cuda")
+    for flags in (0, binding.FLAG_NO_GRAPH, binding.FLAG_NO_LOOKAHEAD):
+        d = src.clone()
+        opt = binding.Options(0, flags, None, 0, ws[offset:].data_ptr(), 4 * (ws.numel() - offset))
+        assert binding.apsp_fw_raw(d.data_ptr(), n, ld, binding.APSP_I32, torch.cuda.current_stream().cuda_stream,
+                                   opt) == binding.APSP_OK
+        torch.cuda.synchronize()
+        assert torch.equal(d, ref)
+        assert bool((ws == 77).all()), flags
