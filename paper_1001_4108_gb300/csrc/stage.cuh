@@ -342,8 +342,8 @@ __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typenam
   }
 }
 
-// rest(b) for int16, two columns per 32-bit word (DPX viaddmin.s16x2): weights
-// are >= 0 and sums fit in 16 bits.  Thread rows st_idx(ty, .), words 2 tx, 2 tx
+// rest(b) for int16, two columns per 32-bit word (DPX viaddmin.s16x2): sums fit
+// in 16 bits, signed.  Thread rows st_idx(ty, .), words 2 tx, 2 tx
 // + 1 (columns 4 tx .. 4 tx + 3).
 template <bool VIA>
 __device__ __forceinline__ void stage_rest_packed(const StageArgs<int16_t> &g, int t, uint32_t *As, uint32_t *Bs,
@@ -404,11 +404,11 @@ __device__ __forceinline__ void stage_rest_packed(const StageArgs<int16_t> &g, i
     if (quad) *reinterpret_cast<uint2 *>(p) = make_uint2(x[a][0], x[a][1]);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int v = (int)(x[a][e / 2] >> (16 * (e % 2)) & 0xffffu);
+      const int16_t v = (int16_t)(x[a][e / 2] >> (16 * (e % 2)) & 0xffffu);
       if (i < g.n && j0 + e < g.n) {
         if (VIA && g.via)
-          note_via(g.via, g.via_ld, i, j0 + e, v, (int)(x0[a][e / 2] >> (16 * (e % 2)) & 0xffffu), b);
-        if (!quad) p[e] = (int16_t)v;
+          note_via(g.via, g.via_ld, i, j0 + e, (int)v, (int)(int16_t)(x0[a][e / 2] >> (16 * (e % 2)) & 0xffffu), b);
+        if (!quad) p[e] = v;
       }
     }
   }
