@@ -284,17 +284,17 @@ APSP_API int64_t apsp_workspace_bytes(int64_t n, int dtype, int32_t kblock);
  * The scratch the packed phase 3 needs (the interleaved row panel) lives in a
  * static device array of the library, 8 MiB, held by every GPU that loads the
  * library until the process exits.  Limit: n <= 16384; larger n returns
- * APSP_EUNSUPPORTED before any device work.  Up to 52 stages of s = 64 the
- * solve runs one head and one rest kernel per stage on the array, in any
- * layout.  Above, with dist 16-byte aligned and ld * 4 a multiple of 16, it
- * always runs the packed kernels on the array (if they cannot run, the call
- * returns APSP_EUNSUPPORTED before any device work); other layouts run the
+ * APSP_EUNSUPPORTED before any device work.  With dist 16-byte aligned, ld * 4
+ * a multiple of 16 and n above one tile, the solve always runs on the array
+ * (up to 52 stages of s = 64 one head and one rest kernel per stage, above the
+ * packed kernels; if they cannot run, the call returns APSP_EUNSUPPORTED
+ * before any device work); other layouts run the
  * unpacked kernels, which need no scratch.  The first call on each device
  * looks up the array's device address (cudaGetSymbolAddress); make that first
  * call before any stream capture.  All calls share the one array and each
  * solve rewrites every part of it that it reads, so nothing needs clearing;
- * calls whose work overlaps on the GPU (e.g. on two streams at once) race on
- * it and must be serialized by the caller.  Launches kernels directly (no
+ * calls that use it and overlap on the GPU (e.g. on two streams at once) race
+ * on it and must be serialized by the caller.  Launches kernels directly (no
  * library-owned graph, stream or workspace).  Stream-ordered like apsp_fw.
  */
 APSP_API int apsp_fw_f32_noalloc(void *dist, int64_t n, int64_t ld, void *stream);

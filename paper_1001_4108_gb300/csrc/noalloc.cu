@@ -73,12 +73,14 @@ extern "C" int apsp_fw_f32_noalloc(void *dist, int64_t n, int64_t ld, void *stre
   a.stream = static_cast<cudaStream_t>(stream);
   a.err = err;
   a.tma_ok = reinterpret_cast<uintptr_t>(dist) % 16 == 0 && ((size_t)ld * sizeof(float)) % 16 == 0;
+  // Rows that are not 16-byte aligned: the kernels that need no scratch, so
+  // that such calls may overlap (the array is one for all calls).
+  if (!a.tma_ok) return apsp::run_f32(a);
   a.ws = panel;
   a.ws_bytes = kPanelFloats * sizeof(float);
   // One panel buffer always fits (s * ceil(n/s) * s floats <= 128 * 16384),
   // so the solve takes the plain schedule on the static array (small ones the
-  // one-head-per-stage schedule, which fits as well); whenever the
-  // layout allows the packed kernels they must use it (the run refuses
+  // one-head-per-stage schedule, which fits as well); it must (the run refuses
   // rather than fall back to the unpacked kernels without telling).
   if (apsp::interleaved_panel_bytes(n, a.S) > a.ws_bytes) return APSP_EUNSUPPORTED;
   a.require_ws = true;

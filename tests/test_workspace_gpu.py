@@ -247,3 +247,28 @@ def test_int32_leaves_a_callers_workspace_alone(n, ld, offset):
         torch.cuda.synchronize()
         assert torch.equal(d, ref)
         assert bool((ws == 77).all()), flags
+
+
+def test_unaligned_noalloc_calls_may_overlap():
+    # rows that are not 16-byte aligned use none of the entry point's shared array
+    n, ld = 1000, 1001
+    srcs = []
+    for k in range(2):
+        srcs.append(torch.zeros((n, ld), device="cuda"))
+        srcs[k][:, :n] = graph("f32", n, k)
+    refs = []
+    for x in srcs:
+        d = x.clone()
+        binding.apsp_fw(d, n, flags=binding.FLAG_NO_WORKSPACE | binding.FLAG_NO_GRAPH)
+        refs.append(d)
+    ss = [torch.cuda.Stream() for _ in range(2)]
+    ds = [x.clone() for x in srcs]
+    torch.cuda.synchronize()
+    for _ in range(5):
+        for k in range(2):
+            with torch.cuda.stream(ss[k]):
+                ds[k].copy_(srcs[k])
+                assert binding.lib().apsp_fw_f32_noalloc(ds[k].data_ptr(), n, ld, ss[k].cuda_stream) == binding.APSP_OK
+        torch.cuda.synchronize()
+        for k in range(2):
+            assert torch.equal(ds[k], refs[k])
