@@ -752,12 +752,14 @@ def measure_single(a, dtype: str, n: int, steps: int, warmup: int, e2e_steps: in
 def roofline_block(dtype: str, n: int, m: dict, sms: int, peaks: dict, peak_kind: str, form_ceiling: float):
     """ALU roofline of the phase-3 launch: relaxations of the launches with a
     full k-block over their summed event durations, against the min-plus
-    peak.  Every candidate d_ik + d_kj needs one 32-bit minimum, and minima
-    run on the ALU pipe: 16 lanes per SM sub-partition, 64 per SM per clock.
-    int32 and fp32: 64 relaxations/clock/SM (a three-input min folds two
-    candidates but retires them at the same rate, measured: forms 4 and 5 of
-    apsp_ubench_minplus); int16x2: two relaxations per DPX lane,
-    128/clock/SM."""
+    reference rate: one relaxation per ALU lane and clock, 16 lanes per SM
+    sub-partition, 64 per SM (int16x2: two per DPX lane, 128).  That is the
+    limit of one minimum per candidate (int32 DPX, int16x2).  For fp32 and
+    int32 it is a yardstick, not a bound: their kernels fold two candidates
+    per three-input min and form sums on the FMA pipe, which in registers
+    alone runs at 72 (fp32, bound by register reads) and 71 (int32) per clock
+    and SM; with the operand loads in the loop, as in form_ceiling, at 62 to
+    64."""
     S = m["cfg"].kblock
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     lanes = 128 if dtype == "i16" else 64
@@ -773,8 +775,11 @@ def roofline_block(dtype: str, n: int, m: dict, sms: int, peaks: dict, peak_kind
             "achieved": achieved, "peak": peak,
             "unit": "relaxations/s", "frac": achieved / peak,
             "peak_basis": f"{sms} SMs x {sm_max:.0f} MHz ({peak_kind} max clock) x {lanes} relaxations "
-                          "per clock per SM (one 32-bit min per candidate on 64 ALU-pipe lanes; "
-                          "int16x2: 2 per DPX lane)",
+                          "per clock per SM (one relaxation per ALU lane; int16x2: 2 per DPX "
+                          "lane).  A reference rate: fp32 and int32 fold two candidates per three-input min "
+                          "and are not bound by it",
+            "form": {"f32": "packed add.f32x2 + three-input min", "i16": "int16x2 DPX add-min",
+                     "i32": "int32 DPX add-min alone (the kernel forms half of its sums on the FMA pipe)"}[dtype],
             "form_ceiling": form_ceiling, "frac_of_form_ceiling": achieved / form_ceiling,
             "traffic": _measured_traffic(dtype, n, S, p3_relax_mean / S ** 3),
             "traffic_source": "ncu dram__bytes_read+write of the same launch kind at n=8192, "

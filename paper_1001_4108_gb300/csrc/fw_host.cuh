@@ -187,7 +187,7 @@ static int run_rounds(const RunArgs &a) {
       return run_dataflow(a, dt, static_cast<int *>(a.ws));
     }
   }
-  // s = 64 without special requests: one launch per stage
+  // s = 64 without special requests: one head and one rest launch per stage
   if constexpr (S == 64) {
     constexpr bool kI16 = std::is_same<T, int16_t>::value;
     constexpr int kType = kI16 ? APSP_I16 : std::is_same<T, float>::value ? APSP_F32 : APSP_I32;

@@ -250,8 +250,15 @@ __device__ __forceinline__ void stage_rest_packed(const StageArgs<int16_t> &g, i
 // rest(b): phase 3 of stage b on the tiles outside rows and columns b, c: CTA t
 // of g.rest updates one 64 x 64 tile, 4 x 4 elements per thread; one more CTA
 // (t = g.rest) moves the closed diagonal tile of stage b to the matrix.  As, Bs:
-// a tile each.  The matrix is read through L2 only: this may start while the
-// launch before it still runs.
+// a tile each.
+// Beside a head, rest(b) waits for nothing before it reads (fw_rest).  That it
+// sees what head(b - 1) and rest(b - 1) wrote: it starts only once every CTA of
+// head(b) has issued launch_dependents, each after its wait_prior_grid; that
+// wait returns when rest(b - 1) has completed and its writes are performed; and
+// rest(b - 1) completes after head(b - 1), for which its last CTA waits.  So
+// all these writes are in L2 before rest(b) starts, and panels and matrix are
+// read from L2 only (bulk copies, ld.cg): an SM's L1 may hold older lines, as
+// launch_dependents by itself orders no memory.
 template <typename T, bool VIA>
 __device__ __forceinline__ void stage_rest(const StageArgs<T> &g, int t, typename Arith<T>::C *As,
                                            typename Arith<T>::C *Bs, uint64_t *bar) {
@@ -692,7 +699,7 @@ __global__ void __launch_bounds__(kStThreads, VIA ? 3 : 4) fw_rest(const StageAr
 // n = 512 fp32 104 with 16, 111 with 32; n = 1920 int32 676 with 32, 727 with
 // 64; n = 2048 int32 779 with 64, 821 with 32, fp32 with unaligned rows 885 and
 // 1071, int16 676 and 594; n = 2304 int16 799 and 840.  In one launch: n = 256 53 (57
-// with two), n = 512 118 (104), n = 1024 323 (221).
+// with two), n = 512 118 (104), n = 1024 323 (227).
 struct HeadCut {
   int W;        // strip width: 16, 32 or 64
   bool merged;  // rest(b) in the head's launch
