@@ -133,7 +133,9 @@ typedef struct apsp_options {
        recorded there, and the phase-3 launch on the call's stream covers every
        tile except row and column r+1 (those run on the internal stream
        before phase 1 of stage r+1, untimed).  Tracing implies
-       APSP_FLAG_NO_GRAPH.  NULL = off. */
+       APSP_FLAG_NO_GRAPH and the lookahead or plain schedule: where an untraced
+       call runs one head and one rest kernel per stage (apsp_config.lookahead),
+       the times are not those of its launches.  NULL = off. */
     void **events;
     int64_t n_events;
     /* Optional device workspace of apsp_workspace_bytes(n, dtype, kblock)
@@ -162,9 +164,13 @@ typedef struct apsp_config {
     int32_t lookahead;       /* 1 if the lookahead schedule is available (stages >= 3,
                                 TMA-staged kernels, library workspace).  With s = 64
                                 and 2 to 52 (fp32), 39 (int32) or 36 (int16) stages,
-                                apsp_fw_paths up to 80, 64 and 64, a call without flags,
-                                tracing or a workspace of its own runs one head and
-                                one rest kernel per stage instead: same results */
+                                apsp_fw_paths up to 80, 64 and 64, a call that forces no
+                                kernel or order (GENERIC, REVERSE_K, NO_LOOKAHEAD,
+                                NO_WORKSPACE, ONE_LAUNCH), is not traced, and has the
+                                library's workspace, or one of its own of (4 R + 2) x
+                                16 KiB (int16 (7 R + 2) x 16 KiB, R = rounds), runs one
+                                head and one rest kernel per stage instead: same
+                                results */
     int32_t strips;          /* 1 if the lookahead and plain schedules on 16-byte
                                 aligned rows cut each 64 x 64 tile of their phase-2
                                 launches (and of the lookahead's cross launches) into
@@ -269,7 +275,8 @@ APSP_API int apsp_path(const void *dist, const int16_t *via, int64_t n, int64_t 
  * buffer runs the plain schedule.  Without a workspace the same results come
  * from slower phase-3 kernels.  The workspaces the library owns can be larger
  * (and int32 solves have one): both panels in copies of their own, at most
- * 4 * s * ceil(n/s) * s * 4 bytes (7 in the place of 4 for int16 with s = 64).
+ * 4 * s * ceil(n/s) * s * 4 bytes (7 in the place of 4 for int16 with s = 64)
+ * and 32 KiB.
  */
 APSP_API int64_t apsp_workspace_bytes(int64_t n, int dtype, int32_t kblock);
 
