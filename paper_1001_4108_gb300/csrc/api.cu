@@ -356,7 +356,8 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
         std::lock_guard<std::mutex> lk(g_mu);
         side_resources_locked(dev, b.stream, cap != cudaStreamCaptureStatusNone, &b);
       }
-      const bool direct = (b.flags & APSP_FLAG_NO_GRAPH) || b.events || cap != cudaStreamCaptureStatusNone;
+      const bool direct =
+          (b.flags & APSP_FLAG_NO_GRAPH) || b.events || cap != cudaStreamCaptureStatusNone || mem.passing();
       st = direct ? run_dtype(b, APSP_I16) : launch_with_graph(b, APSP_I16, dev);
       if (st != APSP_OK) return st;
       if (widen_from_i16(reinterpret_cast<const int16_t *>(buf), ld16, n, static_cast<int32_t *>(dist), ld,
@@ -399,7 +400,9 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   if (via && cudaMemset2DAsync(via, (size_t)via_ld * sizeof(int16_t), 0xff, (size_t)n * sizeof(int16_t), (size_t)n,
                                a.stream) != cudaSuccess)  // every entry -1: never improved
     return APSP_ECUDA;
-  const bool direct = (a.flags & APSP_FLAG_NO_GRAPH) || a.events || cap != cudaStreamCaptureStatusNone;
+  // no graph of a buffer that only this call has
+  const bool direct =
+      (a.flags & APSP_FLAG_NO_GRAPH) || a.events || cap != cudaStreamCaptureStatusNone || lease.passing();
   // Rows that are not 16-byte aligned: the staged kernels work on an aligned
   // copy (two passes over the matrix, against kernels two to four times slower).
   // The one-launch-per-stage schedule takes any layout by itself, at word loads

@@ -35,7 +35,9 @@ class OutsideCapture {
 };
 
 // Device memory in stream order, from one pool per device.  Memory above
-// `keep` bytes goes back to the device when nothing uses it.
+// `keep` bytes goes back to the device when nothing uses it.  What one stream
+// freed is another's only once that work is done: a pool that made the second
+// stream wait would put the two in a row.
 class StreamPool {
  public:
   explicit StreamPool(uint64_t keep) : keep_(keep) {}
@@ -55,8 +57,10 @@ class StreamPool {
       props.location.type = cudaMemLocationTypeDevice;
       props.location.id = dev;
       cudaMemPool_t pool = nullptr;
+      int waits = 0;
       if (!got_memory(cudaMemPoolCreate(&pool, &props)) ||
-          !got_memory(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep_)))
+          !got_memory(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep_)) ||
+          !got_memory(cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &waits)))
         return nullptr;
       pool_[dev] = pool;
     }
@@ -71,6 +75,7 @@ class Workspaces {
   struct Entry {
     int dev;
     unsigned long long id = 0;  // the stream's
+    bool small = false;         // one of those for small buffers only
     std::mutex mu;              // held from take() until the work that uses the buffer is enqueued
     void *p = nullptr;
     size_t bytes = 0;
@@ -110,6 +115,8 @@ class Workspaces {
       entry_.reset();
     }
     explicit operator bool() const { return p != nullptr; }
+    // For this lease only: the next call may get another.
+    bool passing() const { return p && !entry_; }
     void *p = nullptr;
     size_t bytes = 0;
 
@@ -143,7 +150,7 @@ class Workspaces {
     give_back(dev);
     const bool capturing = status == cudaStreamCaptureStatusActive;
     if (const std::shared_ptr<Entry> e =
-            capturing ? captured(dev, stream, capture, graph, bytes, least) : entry(dev, stream)) {
+            capturing ? captured(dev, stream, capture, graph, bytes, least) : entry(dev, stream, bytes)) {
       l.lk_ = std::unique_lock<std::mutex>(e->mu);
       if (e->bytes < bytes && !capturing) {
         if (e->p) forget_(e->p, e->bytes);
@@ -168,12 +175,16 @@ class Workspaces {
   }
 
  private:
-  static constexpr size_t kMaxEntries = 16;
+  // Streams with a buffer of their own: 16, and 48 more for small buffers, the
+  // ones of solves so short that an allocation and a graph captured anew show
+  // (int32 n = 256 on 12 streams 7.6 us a solve; 39 where the last of them were
+  // beyond the entries).
+  static constexpr size_t kMaxEntries = 16, kMaxWithSmall = 64, kSmallBytes = 8u << 20;
   // By the stream's id, not its handle: every thread's cudaStreamPerThread is
   // another stream, and a destroyed stream's handle can come back while its
   // work still runs.  Entries are never evicted: another stream's work may be
   // using the buffer.
-  std::shared_ptr<Entry> entry(int dev, cudaStream_t stream) {
+  std::shared_ptr<Entry> entry(int dev, cudaStream_t stream, size_t bytes) {
     unsigned long long id = 0;
     if (cudaStreamGetId(stream, &id) != cudaSuccess) {
       cudaGetLastError();
@@ -181,11 +192,13 @@ class Workspaces {
     }
     std::lock_guard<std::mutex> lk(mu_);
     for (auto &e : entries_)
-      if (e->dev == dev && e->id == id) return e;
-    if (entries_.size() >= kMaxEntries) return nullptr;
+      if (e->dev == dev && e->id == id) return e->small && bytes > kSmallBytes ? nullptr : e;
+    const bool small = entries_.size() >= kMaxEntries;
+    if (entries_.size() >= kMaxWithSmall || (small && bytes > kSmallBytes)) return nullptr;
     auto e = std::make_shared<Entry>();
     e->dev = dev;
     e->id = id;
+    e->small = small;
     entries_.push_back(e);
     return e;
   }

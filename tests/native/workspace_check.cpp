@@ -222,6 +222,25 @@ static void destroy_graph(unsigned long long id) {
   held.erase(id);
 }
 
+// Streams beyond the first ones keep small buffers, and get large ones for the
+// call.
+static void many_streams() {
+  Workspaces w(forget);
+  std::vector<void *> first;
+  for (int i = 0; i < 40; ++i) first.push_back(w.take(0, stream(i), 1000, 0).p);
+  for (int i = 0; i < 40; ++i) {
+    Workspaces::Lease l = w.take(0, stream(i), 1000, 0);
+    check(l.p == first[i] && !l.passing(), "a stream's small buffer stays");
+  }
+  const size_t before = used;
+  for (int i = 30; i < 50; ++i) {
+    Workspaces::Lease l = w.take(0, stream(i), 9 << 20, 0);
+    check(l && l.passing(), "a large buffer beyond the first streams is for the call");
+  }
+  check(used == before, "and given back after it");
+  check(w.take(0, stream(30), 1000, 0).p == first[30], "beside the stream's small one");
+}
+
 // Stream captures: buffers of their own, that live as long as the graph.
 static void captures() {
   Workspaces w(forget);
@@ -286,6 +305,7 @@ int main() {
   reuse_and_growth();
   out_of_memory();
   captures();
+  many_streams();
   stream_identity();
   threads();
   std::printf(fails ? "%d failed checks\n" : "ok\n", fails);
