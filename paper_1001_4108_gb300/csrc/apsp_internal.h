@@ -103,7 +103,9 @@ inline bool uses_strips(int S, int R, bool f32, bool i16) {
 // is further behind: fp32 n = 2304 1864 and 1276, 3072 3605 and 2562, 4096 6865
 // and 5681; int32 2304 1673 and 1208, 3072 2906 and 2468, 3584 4323 and 3774,
 // 4032 6383 and 5377; int16 2560 1397 and 1153, 3072 1980 and 1775, 4032 3827 and
-// 3632; fp32 5056 (79 stages) 10477 and 9482.
+// 3632; fp32 5056 (79 stages) 10477 and 9482.  All of solves alone on the GPU:
+// side by side they pay for the heads' redundant closures (int32 n = 1024 on 4
+// streams 99 and 122 us a solve).
 inline int stage_max_rounds(bool f32, bool i16, bool via) {
   return via ? (f32 ? 80 : 64) : (f32 ? 52 : i16 ? 36 : 39);
 }
