@@ -318,9 +318,9 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   const size_t es = (size_t)elem_size(dtype);
   a.tma_ok = (reinterpret_cast<uintptr_t>(dist) % 16 == 0) && ((size_t)ld * es) % 16 == 0;
 
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(a.stream, &cap) != cudaSuccess) return APSP_ECUDA;
-  if (cap != cudaStreamCaptureStatusNone && (a.flags & (APSP_FLAG_VALIDATE | APSP_FLAG_NEGCYCLE)))
+  Capture cap;
+  if (!capture_of(a.stream, &cap)) return APSP_ECUDA;
+  if (cap.active && (a.flags & (APSP_FLAG_VALIDATE | APSP_FLAG_NEGCYCLE)))
     return APSP_EINVAL;  // both synchronize the stream
   const bool narrow = dtype == APSP_I32 && (a.flags & APSP_FLAG_NARROW);
   if (narrow && (via || (opt && opt->workspace))) return APSP_EINVAL;
@@ -339,7 +339,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
     const bool staged = uses_stage_launches(S16, R16, APSP_I16, false, a.flags, a.events != nullptr);
     const size_t ws16 = staged ? std::max(least16, stage_ws_bytes(R16, true)) : least16;
     Workspaces::Lease mem =
-        g_workspaces.take(dev, a.stream, copy_bytes + ws16, copy_bytes + least16);
+        g_workspaces.take(dev, a.stream, cap, copy_bytes + ws16, copy_bytes + least16);
     if (mem) {  // else: the int32 path, same result
       char *buf = static_cast<char *>(mem.p);
       if (narrow_to_i16(static_cast<const int32_t *>(dist), n, ld, reinterpret_cast<int16_t *>(buf), ld16,
@@ -354,10 +354,10 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       b.ws = b.ws_bytes ? buf + copy_bytes : nullptr;
       if (!(b.flags & APSP_FLAG_NO_LOOKAHEAD)) {
         std::lock_guard<std::mutex> lk(g_mu);
-        side_resources_locked(dev, b.stream, cap != cudaStreamCaptureStatusNone, &b);
+        side_resources_locked(dev, b.stream, cap.active, &b);
       }
       const bool direct =
-          (b.flags & APSP_FLAG_NO_GRAPH) || b.events || cap != cudaStreamCaptureStatusNone || mem.passing();
+          (b.flags & APSP_FLAG_NO_GRAPH) || b.events || cap.active || mem.passing();
       st = direct ? run_dtype(b, APSP_I16) : launch_with_graph(b, APSP_I16, dev);
       if (st != APSP_OK) return st;
       if (widen_from_i16(reinterpret_cast<const int16_t *>(buf), ld16, n, static_cast<int32_t *>(dist), ld,
@@ -389,20 +389,20 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
       if (dtype == APSP_I32) a.ws_bytes = std::min(a.ws_bytes, need);
     }
   } else if (need || more) {
-    lease = g_workspaces.take(dev, a.stream, std::max(need, more), need);
+    lease = g_workspaces.take(dev, a.stream, cap, std::max(need, more), need);
     a.ws = lease.p;  // none: the kernels fall back to the form that needs none
     a.ws_bytes = lease.bytes;
   }
   if (!(a.flags & APSP_FLAG_NO_LOOKAHEAD)) {
     std::lock_guard<std::mutex> lk(g_mu);
-    side_resources_locked(dev, a.stream, cap != cudaStreamCaptureStatusNone, &a);
+    side_resources_locked(dev, a.stream, cap.active, &a);
   }
   if (via && cudaMemset2DAsync(via, (size_t)via_ld * sizeof(int16_t), 0xff, (size_t)n * sizeof(int16_t), (size_t)n,
                                a.stream) != cudaSuccess)  // every entry -1: never improved
     return APSP_ECUDA;
   // no graph of a buffer that only this call has
   const bool direct =
-      (a.flags & APSP_FLAG_NO_GRAPH) || a.events || cap != cudaStreamCaptureStatusNone || lease.passing();
+      (a.flags & APSP_FLAG_NO_GRAPH) || a.events || cap.active || lease.passing();
   // Rows that are not 16-byte aligned: the staged kernels work on an aligned
   // copy (two passes over the matrix, against kernels two to four times slower).
   // The one-launch-per-stage schedule takes any layout by itself, at word loads
@@ -416,7 +416,7 @@ int solve(void *dist, int64_t n, int64_t ld, int dtype, const apsp_options *opt,
   const bool any_layout = staged && a.ws_bytes >= more && R < kStageCopyRounds;
   void *copy = nullptr;
   const int64_t cld = (n * (int64_t)es + 15) / 16 * 16 / (int64_t)es;
-  if (!a.tma_ok && !any_layout && R > 1 && !(a.flags & kInPlace) && cap == cudaStreamCaptureStatusNone &&
+  if (!a.tma_ok && !any_layout && R > 1 && !(a.flags & kInPlace) && !cap.active &&
       a.stream != cudaStreamPerThread)  // see Workspaces::take
     copy = g_copies.alloc(dev, (size_t)n * cld * es, a.stream);
   if (copy) {

@@ -34,6 +34,24 @@ class OutsideCapture {
   cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
 };
 
+// Whether a stream is being captured, and into which graph (nullptr: the
+// capture is invalid).
+struct Capture {
+  bool active = false;
+  unsigned long long id = 0;
+  cudaGraph_t graph = nullptr;
+};
+inline bool capture_of(cudaStream_t stream, Capture *c) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamGetCaptureInfo(stream, &status, &c->id, &c->graph, nullptr, nullptr, nullptr) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  c->active = status != cudaStreamCaptureStatusNone;
+  if (status != cudaStreamCaptureStatusActive) c->graph = nullptr;
+  return true;
+}
+
 // Device memory in stream order, from one pool per device.  Memory above
 // `keep` bytes goes back to the device when nothing uses it.  What one stream
 // freed is another's only once that work is done: a pool that made the second
@@ -130,29 +148,20 @@ class Workspaces {
   // forget(p, bytes): called before that buffer is freed
   explicit Workspaces(void (*forget)(void *, size_t)) : forget_(forget) {}
 
-  // At least `bytes` bytes for work on `stream`, else at least `least` (if not
+  // At least `bytes` bytes for work on `stream` (capture_of it), else at least `least` (if not
   // 0), else an empty lease: there is no memory.  The caller then runs kernels
   // that need less or none.
   // Nothing is allocated or freed in the order of cudaStreamPerThread, which
   // ends with its thread: a thread that ended with such frees pending left a
   // later device synchronize waiting.
-  Lease take(int dev, cudaStream_t stream, size_t bytes, size_t least) {
+  Lease take(int dev, cudaStream_t stream, const Capture &cap, size_t bytes, size_t least) {
     Lease l;
     l.stream_ = stream;
-    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-    unsigned long long capture = 0;
-    cudaGraph_t graph = nullptr;
-    if (cudaStreamGetCaptureInfo(stream, &status, &capture, &graph, nullptr, nullptr, nullptr) != cudaSuccess ||
-        status == cudaStreamCaptureStatusInvalidated) {
-      cudaGetLastError();
-      return l;
-    }
     give_back(dev);
-    const bool capturing = status == cudaStreamCaptureStatusActive;
     if (const std::shared_ptr<Entry> e =
-            capturing ? captured(dev, stream, capture, graph, bytes, least) : entry(dev, stream, bytes)) {
+            cap.active ? captured(dev, stream, cap, bytes, least) : entry(dev, stream, bytes)) {
       l.lk_ = std::unique_lock<std::mutex>(e->mu);
-      if (e->bytes < bytes && !capturing) {
+      if (e->bytes < bytes && !cap.active) {
         if (e->p) forget_(e->p, e->bytes);
         if (stream == cudaStreamPerThread) {
           replace_outside(e.get(), bytes, least);
@@ -168,7 +177,7 @@ class Workspaces {
       } else {
         l.lk_.unlock();
       }
-    } else if (!capturing && stream != cudaStreamPerThread) {
+    } else if (!cap.active && stream != cudaStreamPerThread) {
       l.bytes = alloc(pool_, dev, stream, bytes, least, &l.p);  // more streams than entries: for this call
     }
     return l;
@@ -204,18 +213,18 @@ class Workspaces {
   }
   // The buffer of the solves that are captured on `stream` into `graph`, one
   // after the other; nullptr without memory.
-  std::shared_ptr<Entry> captured(int dev, cudaStream_t stream, unsigned long long capture, cudaGraph_t graph,
-                                  size_t bytes, size_t least) {
+  std::shared_ptr<Entry> captured(int dev, cudaStream_t stream, const Capture &cap, size_t bytes, size_t least) {
+    if (!cap.graph) return nullptr;
     std::lock_guard<std::mutex> lk(mu_);
     for (auto &e : captured_)
-      if (e->capture == capture && e->stream == stream && e->dev == dev && e->bytes >= bytes) return e;
+      if (e->capture == cap.id && e->stream == stream && e->dev == dev && e->bytes >= bytes) return e;
     const OutsideCapture guard;
     const cudaStream_t home = home_stream(dev);
     if (!home) return nullptr;
     auto e = std::make_shared<Entry>();
     e->dev = dev;
     e->stream = stream;
-    e->capture = capture;
+    e->capture = cap.id;
     if (!(e->bytes = alloc(outside_, dev, home, bytes, least, &e->p))) return nullptr;
     auto *held = new std::shared_ptr<Entry>(e);
     cudaUserObject_t object = nullptr;
@@ -224,7 +233,7 @@ class Workspaces {
     if (!made) delete held;
     // the memory is there before any launch of the graph
     if (!made || cudaStreamSynchronize(home) != cudaSuccess ||
-        cudaGraphRetainUserObject(graph, object, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+        cudaGraphRetainUserObject(cap.graph, object, 1, cudaGraphUserObjectMove) != cudaSuccess) {
       cudaGetLastError();
       if (made) cudaUserObjectRelease(object, 1);
       cudaFreeAsync(e->p, home);
@@ -236,6 +245,7 @@ class Workspaces {
   // A larger buffer for a calling thread's own stream; it waits for that
   // stream's work with the old one.
   void replace_outside(Entry *e, size_t bytes, size_t least) {
+    const OutsideCapture guard;
     if (e->p && cudaStreamSynchronize(cudaStreamPerThread) != cudaSuccess) return;
     std::lock_guard<std::mutex> lk(mu_);
     const cudaStream_t home = home_stream(e->dev);

@@ -136,20 +136,26 @@ cudaError_t cudaGetLastError() {
 }
 }
 
+static Workspaces::Lease take(Workspaces &w, int dev, cudaStream_t s, size_t bytes, size_t least) {
+  apsp::Capture c;
+  check(apsp::capture_of(s, &c), "a stream's capture state");
+  return w.take(dev, s, c, bytes, least);
+}
+
 static void reuse_and_growth() {
   Workspaces w(forget);
   void *a = nullptr;
   {
-    Workspaces::Lease l = w.take(0, stream(1), 1000, 0);
+    Workspaces::Lease l = take(w, 0, stream(1), 1000, 0);
     check(l && l.bytes == 1000, "a first buffer");
     a = l.p;
   }
-  check(w.take(0, stream(1), 500, 0).p == a, "a smaller request reuses it");
-  check(w.take(0, stream(2), 500, 0).p != a, "another stream has its own");
-  check(w.take(1, stream(1), 500, 0).p != a, "so has another device");
-  check(w.take(0, stream(1), 2000, 0).bytes == 2000, "a larger request");
+  check(take(w, 0, stream(1), 500, 0).p == a, "a smaller request reuses it");
+  check(take(w, 0, stream(2), 500, 0).p != a, "another stream has its own");
+  check(take(w, 1, stream(1), 500, 0).p != a, "so has another device");
+  check(take(w, 0, stream(1), 2000, 0).bytes == 2000, "a larger request");
   check(forgotten.count(a) == 1, "graphs that use the old buffer are dropped");
-  for (int i = 3; i < 40; ++i) w.take(0, stream(i), 1000 * i, 0);
+  for (int i = 3; i < 40; ++i) take(w, 0, stream(i), 1000 * i, 0);
   check(syncs == 0, "growing buffers and many streams synchronize the device");
 }
 
@@ -157,32 +163,32 @@ static void reuse_and_growth() {
 static void out_of_memory() {
   Workspaces w(forget);
   const size_t before = limit;
-  check((bool)w.take(0, stream(1), 100, 0), "a small buffer");
+  check((bool)take(w, 0, stream(1), 100, 0), "a small buffer");
   limit = used + 400;
-  check(w.take(0, stream(1), 1000, 300).bytes == 300, "no memory for a larger one: the smaller size");
+  check(take(w, 0, stream(1), 1000, 300).bytes == 300, "no memory for a larger one: the smaller size");
   check(last_error == cudaSuccess, "a failed allocation leaves an error for the launch checks");
-  check(!w.take(0, stream(1), 2000, 1000), "no memory");
+  check(!take(w, 0, stream(1), 2000, 1000), "no memory");
   limit = used;
-  check(!w.take(0, stream(2), 1, 0) && last_error == cudaSuccess, "no memory on a new stream");
+  check(!take(w, 0, stream(2), 1, 0) && last_error == cudaSuccess, "no memory on a new stream");
   limit = before;
-  check(w.take(0, stream(2), 1, 0).bytes == 1, "a later call finds memory");
+  check(take(w, 0, stream(2), 1, 0).bytes == 1, "a later call finds memory");
 }
 
 // One handle, several streams: each has its own buffer.
 static void stream_identity() {
   Workspaces w(forget);
-  Workspaces::Lease mine = w.take(0, cudaStreamPerThread, 1000, 0);
+  Workspaces::Lease mine = take(w, 0, cudaStreamPerThread, 1000, 0);
   void *other = nullptr;
-  std::thread([&] { other = w.take(0, cudaStreamPerThread, 1000, 0).p; }).join();
+  std::thread([&] { other = take(w, 0, cudaStreamPerThread, 1000, 0).p; }).join();
   check(mine && other && other != mine.p, "two threads' cudaStreamPerThread share a buffer");
   mine.release();
-  check(w.take(0, cudaStreamPerThread, 5000, 0).bytes == 5000, "and can grow");
-  for (int i = 0; i < 20; ++i) std::thread([&] { w.take(0, cudaStreamPerThread, 1000, 0); }).join();
+  check(take(w, 0, cudaStreamPerThread, 5000, 0).bytes == 5000, "and can grow");
+  for (int i = 0; i < 20; ++i) std::thread([&] { take(w, 0, cudaStreamPerThread, 1000, 0); }).join();
   check(per_thread_order == 0, "memory in the order of a thread's own stream");
   Workspaces v(forget);
-  void *a = v.take(0, stream(1), 1000, 0).p;
+  void *a = take(v, 0, stream(1), 1000, 0).p;
   ++recreated[stream(1)];
-  check(v.take(0, stream(1), 1000, 0).p != a, "a new stream has the buffer of a destroyed one of that handle");
+  check(take(v, 0, stream(1), 1000, 0).p != a, "a new stream has the buffer of a destroyed one of that handle");
 }
 
 // Threads: while one holds a lease, its buffer is neither freed nor handed to
@@ -192,7 +198,7 @@ static void threads() {
   std::atomic<int> freed{0}, shared{0}, none{0};
   auto client = [&](int t, int s) {
     for (int i = 0; i < 200; ++i) {
-      Workspaces::Lease l = w.take(0, stream(s), 100 + 37 * ((i + t) % 5) * (1 + i / 20), 0);
+      Workspaces::Lease l = take(w, 0, stream(s), 100 + 37 * ((i + t) % 5) * (1 + i / 20), 0);
       if (!l) {
         ++none;
         continue;
@@ -227,59 +233,59 @@ static void destroy_graph(unsigned long long id) {
 static void many_streams() {
   Workspaces w(forget);
   std::vector<void *> first;
-  for (int i = 0; i < 40; ++i) first.push_back(w.take(0, stream(i), 1000, 0).p);
+  for (int i = 0; i < 40; ++i) first.push_back(take(w, 0, stream(i), 1000, 0).p);
   for (int i = 0; i < 40; ++i) {
-    Workspaces::Lease l = w.take(0, stream(i), 1000, 0);
+    Workspaces::Lease l = take(w, 0, stream(i), 1000, 0);
     check(l.p == first[i] && !l.passing(), "a stream's small buffer stays");
   }
   const size_t before = used;
   for (int i = 30; i < 50; ++i) {
-    Workspaces::Lease l = w.take(0, stream(i), 9 << 20, 0);
+    Workspaces::Lease l = take(w, 0, stream(i), 9 << 20, 0);
     check(l && l.passing(), "a large buffer beyond the first streams is for the call");
   }
   check(used == before, "and given back after it");
-  check(w.take(0, stream(30), 1000, 0).p == first[30], "beside the stream's small one");
+  check(take(w, 0, stream(30), 1000, 0).p == first[30], "beside the stream's small one");
 }
 
 // Stream captures: buffers of their own, that live as long as the graph.
 static void captures() {
   Workspaces w(forget);
   forgotten.clear();
-  void *own = w.take(0, stream(1), 1000, 0).p;
+  void *own = take(w, 0, stream(1), 1000, 0).p;
   capturing[stream(1)] = 1;
-  void *a = w.take(0, stream(1), 1000, 0).p;
+  void *a = take(w, 0, stream(1), 1000, 0).p;
   check(a && a != own, "a capture does not get the stream's buffer");
-  check(w.take(0, stream(1), 800, 0).p == a, "the next solve of that capture shares its buffer");
-  void *b = w.take(0, stream(1), 3000, 0).p;
+  check(take(w, 0, stream(1), 800, 0).p == a, "the next solve of that capture shares its buffer");
+  void *b = take(w, 0, stream(1), 3000, 0).p;
   check(b && b != a && live.count(a), "a larger one gets another, and the first stays");
   capturing[stream(2)] = 1;  // forked in the same capture: runs beside it
-  void *c = w.take(0, stream(2), 1000, 0).p;
+  void *c = take(w, 0, stream(2), 1000, 0).p;
   check(c && c != a && c != b, "two streams of one capture have their own");
   capturing.clear();
   capturing[stream(1)] = 2;
-  void *d = w.take(0, stream(1), 1000, 0).p;
+  void *d = take(w, 0, stream(1), 1000, 0).p;
   check(d && d != a && d != own, "two captures on one stream have their own");
   capturing.clear();
-  check(w.take(0, stream(1), 1000, 0).p == own, "outside the captures, the stream's own");
-  for (int i = 1; i < 30; ++i) w.take(0, stream(i), 100000, 0);
+  check(take(w, 0, stream(1), 1000, 0).p == own, "outside the captures, the stream's own");
+  for (int i = 1; i < 30; ++i) take(w, 0, stream(i), 100000, 0);
   check(!live.count(own) && live.count(a) && live.count(b) && live.count(c) && live.count(d),
         "larger solves and other streams leave the captures' buffers alone");
   check(forgotten.count(a) + forgotten.count(b) + forgotten.count(c) + forgotten.count(d) == 0,
         "the library's graphs have no part in them");
   destroy_graph(1);
-  w.take(0, stream(1), 1, 0);
+  take(w, 0, stream(1), 1, 0);
   check(!live.count(a) && !live.count(b) && !live.count(c) && live.count(d), "gone with their graph");
   destroy_graph(2);
-  w.take(0, stream(1), 1, 0);
+  take(w, 0, stream(1), 1, 0);
   check(!live.count(d), "and the last");
   // no memory, or a graph that takes no objects: no buffer, none left behind
   const size_t before = limit, was = used;
   capturing[stream(3)] = 3;
   limit = used;
-  check(!w.take(0, stream(3), 1000, 100), "no memory in a capture");
+  check(!take(w, 0, stream(3), 1000, 100), "no memory in a capture");
   limit = before;
   refuse_objects = true;
-  check(!w.take(0, stream(3), 1000, 100), "an object that the graph refuses");
+  check(!take(w, 0, stream(3), 1000, 100), "an object that the graph refuses");
   refuse_objects = false;
   check(used == was && last_error == cudaSuccess, "nothing is left of either");
   capturing.clear();
