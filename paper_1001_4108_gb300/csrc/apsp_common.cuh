@@ -67,7 +67,8 @@ template <> struct Arith<int16_t> {
 // executes, and one three-input min; a tile product that takes half of its
 // elements each way spreads over both pipes: 61.4 relaxations per clock and
 // SM against 57.3 with DPX only (4 x 4 elements per thread, operands in
-// shared memory; a loop of its own, not a form of apsp_ubench_minplus).  `one` is a runtime value so that the multiplication stays.
+// shared memory; a loop of its own, not a form of apsp_ubench_minplus).
+// `one` is a runtime value so that the multiplication stays.
 __device__ __forceinline__ float min3f(float a, float b, float c) {
   float r;
   asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
