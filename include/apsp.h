@@ -148,8 +148,9 @@ typedef struct apsp_options {
        allocated on first use.  A solve in a stream capture gets a buffer that
        belongs to the captured graph (shared by the solves captured on one
        stream in it) and is given back when the graph and what was made from
-       it are destroyed: captured graphs share none of it with each other or
-       with later calls, and can be launched on any stream. */
+       it are destroyed: captures share none of it with each other or with
+       later calls, and their graphs can be launched on any stream (executables
+       of one and the same graph one after the other: they solve one matrix). */
     void *workspace;
     int64_t workspace_bytes;
 } apsp_options;
